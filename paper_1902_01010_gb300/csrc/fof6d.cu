@@ -5,7 +5,7 @@
 // candidate, lx is the 3D linking length and lv = alpha_v sigma_v per halo.
 //
 // GB300 design: candidates (ell >= ell_th, or all members) are compacted per halo in the
-// halo's Morton order, so 32 consecutive candidates form a compact "tile" with an integer
+// halo's Hilbert order, so 32 consecutive candidates form a compact "tile" with an integer
 // bounding box. One warp owns one tile and walks the later tiles of its halo, 32 box
 // tests at a time across the lanes: a box gap of at least the spatial linking length
 // skips a tile pair outright; otherwise the 32 x 32 pairs are tested from shared memory. The predicate is FP64 with every operation rounded

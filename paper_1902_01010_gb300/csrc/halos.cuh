@@ -6,7 +6,7 @@ namespace vr {
 
 // Halos are 3D groups with at least nmin members (Sec. 2.2, N >= N_min), numbered in
 // increasing label order. Members are stored per halo in one contiguous run of "slots",
-// ordered by the Morton code of their unwrapped position inside the halo's bounding box
+// ordered along a space-filling curve by their unwrapped position inside the halo's bounding box
 // (spatial locality for the neighbour searches).
 struct HaloSeg {
   int64_t n = 0;       // particles
@@ -25,11 +25,12 @@ struct HaloSeg {
 
 // Carves and builds the segmentation (one stream synchronisation to read H and NHP).
 // The outputs take halo_seg_bytes(n, nmin) and stay; the build needs a further
-// halo_seg_temp_bytes(n, nmin), released (arena offset restored) on return.
+// halo_seg_temp_bytes(n, nmin), released (arena offset restored) on return. `hilbert`:
+// members along the Hilbert curve (the linkers), else the Morton curve (f_l and after).
 size_t halo_seg_bytes(int64_t n, int nmin);
 size_t halo_seg_temp_bytes(int64_t n, int nmin);
 vr_status build_halos(vr_ctx *ctx, const int32_t *pos, const float *vel, int64_t n,
-                      const int32_t *label, int nmin, int nsmall, Arena &ar, cudaStream_t s,
+                      const int32_t *label, int nmin, bool hilbert, Arena &ar, cudaStream_t s,
                       HaloSeg *out);
 
 }  // namespace vr

@@ -75,7 +75,7 @@ vr_status vr_velden(vr_ctx *ctx, const int32_t *pos, const float *vel, int64_t n
   HaloSeg g;
   st = fill_f32(ctx, f_l, n, NAN, s);
   if (st != VR_OK) return st;
-  st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g);
+  st = build_halos(ctx, pos, vel, n, label, p->nmin, false, ar, s, &g);
   if (st != VR_OK) return st;
   return run_velden(ctx, g, p, ar, f_l, s);
 }
@@ -97,7 +97,7 @@ vr_status vr_outlier_ratio(vr_ctx *ctx, const int32_t *pos, const float *vel, co
   HaloSeg g;
   if ((st = fill_f32(ctx, R, n, NAN, s)) != VR_OK) return st;
   if ((st = fill_f32(ctx, ell, n, NAN, s)) != VR_OK) return st;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, false, ar, s, &g)) != VR_OK) return st;
   Background bg;
   if ((st = run_background(ctx, g, p, ar, f_l, R, halo_stats, &bg, s)) != VR_OK) return st;
   if ((st = run_fit(ctx, g, bg, p, R, halo_stats, ell, s)) != VR_OK) return st;
@@ -120,7 +120,7 @@ vr_status vr_fof6d(vr_ctx *ctx, const int32_t *pos, const float *vel, const floa
   if ((st = ws_upfront(ctx, n, p, ws_bytes)) != VR_OK) return st;
   HaloSeg g;
   if ((st = fill_i32(ctx, label6, n, -1, s)) != VR_OK) return st;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, true, ar, s, &g)) != VR_OK) return st;
   if (nhalo != g.H)
     return set_error(ctx, VR_ERR_INVALID_ARG, "nhalo = %lld but the labels define %lld halos",
                      (long long)nhalo, (long long)g.H);
@@ -145,7 +145,7 @@ vr_status vr_fof6d_field(vr_ctx *ctx, const int32_t *pos, const float *vel, int6
   if ((st = ws_upfront(ctx, n, p, ws_bytes)) != VR_OK) return st;
   HaloSeg g;
   if ((st = fill_i32(ctx, label6, n, -1, s)) != VR_OK) return st;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, true, ar, s, &g)) != VR_OK) return st;
   if ((st = run_halo_frame(ctx, g, p->nsearch_min, halo_stats, s)) != VR_OK) return st;
   if ((st = field_lengths(ctx, g.H, lx * lx, alpha_v, halo_stats, s)) != VR_OK) return st;
   vr_params q = *p;
@@ -184,7 +184,7 @@ vr_status vr_grow_groups(vr_ctx *ctx, const int32_t *pos, const float *vel, cons
   Arena ar(ws, ws_bytes);
   if ((st = ws_upfront(ctx, n, p, ws_bytes)) != VR_OK) return st;
   HaloSeg g;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, true, ar, s, &g)) != VR_OK) return st;
   if (nhalo != g.H)
     return set_error(ctx, VR_ERR_INVALID_ARG, "nhalo = %lld but the labels define %lld halos",
                      (long long)nhalo, (long long)g.H);
@@ -221,7 +221,7 @@ vr_status vr_core_search(vr_ctx *ctx, const int32_t *pos, const float *vel, int6
   Arena ar(ws, ws_bytes);
   if ((st = ws_upfront(ctx, n, p, ws_bytes)) != VR_OK) return st;
   HaloSeg g;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, true, ar, s, &g)) != VR_OK) return st;
   if ((st = run_halo_frame(ctx, g, p->nsearch_min, halo_stats, s)) != VR_OK) return st;
   if ((st = run_cores(ctx, g, p, cp, lx, alpha_v, ar, label6, halo_stats, core, level, ncores,
                       s)) != VR_OK)
@@ -259,7 +259,7 @@ vr_status vr_core_grow(vr_ctx *ctx, const int32_t *pos, const float *vel, int64_
   Arena ar(ws, ws_bytes);
   if ((st = ws_upfront(ctx, n, p, ws_bytes)) != VR_OK) return st;
   HaloSeg g;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, true, ar, s, &g)) != VR_OK) return st;
   if ((st = run_halo_frame(ctx, g, p->nsearch_min, halo_stats, s)) != VR_OK) return st;
   CoreExtra ex;
   ex.searched = ar.take<int32_t>(n);
@@ -313,7 +313,7 @@ vr_status vr_find_substructure(vr_ctx *ctx, const int32_t *pos, const float *vel
   if ((st = fill_f32(ctx, R, n, NAN, s)) != VR_OK) return st;
   if ((st = fill_f32(ctx, ell, n, NAN, s)) != VR_OK) return st;
   if ((st = fill_i32(ctx, label6, n, -1, s)) != VR_OK) return st;
-  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, p->nse, ar, s, &g)) != VR_OK) return st;
+  if ((st = build_halos(ctx, pos, vel, n, label, p->nmin, false, ar, s, &g)) != VR_OK) return st;
   std::vector<uint32_t> hoff_host;
   if (plain && g.H > 0) {
     hoff_host.resize(g.H + 1);
