@@ -140,14 +140,10 @@ __device__ __forceinline__ bool link6(long long dx2, float4 a, float4 b, const L
   return true;
 }
 
-// One warp per tile i: pairs with every later tile of the same halo (and inside tile i).
-// The lanes test the boxes of 32 later tiles at once; each tile that comes within the
-// spatial linking length is staged in shared memory and its 32 members are read back by
-// every lane. The predicate is first evaluated in FP32 with every operand a rounded copy
-// of the FP64 one: its relative error is below 8 * 2^-24 < 5e-7, so a result outside
-// [1 - 1e-5, 1 + 1e-5] decides the FP64 comparison too; pairs inside that band, and every
-// pair when V_r / Theta_op are on, take the exact FP64 path. The FP32 route is used only
-// when lx2 and lv2 are normal FP32 numbers.
+// The linker's walk. One warp per tile i: the pairs inside tile i, and those with every
+// later tile of the same halo whose box comes within the spatial linking length (the lanes
+// test the boxes of 32 later tiles at once; a tile that passes is staged in shared memory
+// and its members are read back by every lane).
 //
 // The same walk serves the relaxed pass of the two-stage linking (MODE > 0, lx2 scaled
 // by gamma_x^2): MODE 1 unites linked pairs of untagged candidates, MODE 2 counts links
@@ -184,6 +180,160 @@ __device__ __forceinline__ void hash_add(const GrowArgs &G, u64 key) {
   raise_error(G.st, VR_ERR_UNSUPPORTED, 5);
 }
 
+// What decides a link in one halo. The predicate is evaluated in FP32 first, with an error
+// bound, and in FP64 only where the FP32 value does not settle it: the FP64 rate of the
+// GB300 is a small fraction of its FP32 rate, and one exact evaluation costs two FP64
+// divisions and, with V_r / Theta_op, some forty further operations.
+struct LinkC {
+  Link6 L;
+  long long T;          // ceil(lx2): dx2 < lx2 <=> dx2 < T for whole dx2
+  float ilx2, ilv2;     // 1 / lx2, 1 / lv2 (when fast)
+  float v0, v1, v2, E;  // halo velocity, and the rounding error of one of its components
+  float vr2, c;         // V_r^2, cos(Theta_op)
+  bool fast;            // lx2 and lv2 are normal FP32 numbers
+};
+
+__device__ __forceinline__ LinkC link_consts(const double *row, double gx, double vr2, double cos2,
+                                             int use_lv, int use_vt) {
+  LinkC c;
+  Link6 &L = c.L;
+  L.lx2 = __dmul_rn(__dmul_rn(row[VR_H_LX2], gx), gx);  // gx = 1 leaves lx2 as it is
+  L.lv2 = row[VR_H_LV2];
+  L.vf0 = row[VR_H_VFX];
+  L.vf1 = row[VR_H_VFY];
+  L.vf2 = row[VR_H_VFZ];
+  L.vr2 = vr2;
+  L.cos2 = cos2;
+  L.use_lv = use_lv;
+  L.use_vt = use_vt;
+  // NaN and lx2 <= 0 link nothing (T = 0)
+  c.T = L.lx2 > 0.0 ? (L.lx2 < 4e18 ? (long long)ceil(L.lx2) : 0x7fffffffffffffffLL) : 0;
+  c.fast = L.lx2 > 1e-30 && L.lx2 < 1e30 && (!use_lv || (L.lv2 > 1e-30 && L.lv2 < 1e30));
+  c.ilx2 = c.fast ? (float)(1.0 / L.lx2) : 0.0f;
+  c.ilv2 = c.fast && use_lv ? (float)(1.0 / L.lv2) : 0.0f;
+  c.v0 = (float)L.vf0;
+  c.v1 = (float)L.vf1;
+  c.v2 = (float)L.vf2;
+  c.E = 5.9604645e-8f * fmaxf(fabsf(c.v0), fmaxf(fabsf(c.v1), fabsf(c.v2)));
+  c.vr2 = (float)vr2;
+  c.c = (float)sqrt(cos2);
+  return c;
+}
+
+// s = |v - vf|^2 in FP32 and a bound on the relative error that u = v - vf carries into s
+// and into a dot product (sqrt(3) E per vector from the rounded vf, 2^-24 per operation).
+__device__ __forceinline__ void frame_len(const LinkC &c, float4 q, float &s, float &rel) {
+  const float x = q.x - c.v0, y = q.y - c.v1, z = q.z - c.v2;
+  s = x * x + y * y + z * z;
+  rel = 4.0f * c.E * rsqrtf(s) + 1e-6f;
+}
+
+// The predicate for members a and b: fa, fb positions as FP32 (whole numbers below 2^23,
+// so every difference is exact), qa, qb velocities, (s, r) from frame_len (used with
+// V_r / Theta_op only). FP32 errors: q below 8 * 2^-24 < 5e-7 relative, decided outside
+// [1 - 1e-5, 1 + 1e-5]; the V_r and Theta_op tests within ra + rb. NaN settles nothing and
+// goes to FP64.
+__device__ __forceinline__ bool pair_link(const LinkC &c, float4 fa, float4 qa, float sa, float ra,
+                                          float4 fb, float4 qb, float sb, float rb) {
+  const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;
+  if (c.fast) {
+    float q = (dx * dx + dy * dy + dz * dz) * c.ilx2;
+    if (c.L.use_lv) {
+      const float d0 = qa.x - qb.x, d1 = qa.y - qb.y, d2 = qa.z - qb.z;
+      q += (d0 * d0 + d1 * d1 + d2 * d2) * c.ilv2;
+    }
+    if (q >= 1.0f + 1e-5f) return false;
+    if (q <= 1.0f - 1e-5f) {
+      if (!c.L.use_vt) return true;
+      const float e = ra + rb;
+      if (sa > 1e-15f && sa < 1e15f && sb > 1e-15f && sb < 1e15f && e < 0.5f) {
+        const float ka = c.vr2 * sb, kb = c.vr2 * sa;
+        if (sa > ka * (1.0f + e) || sb > kb * (1.0f + e)) return false;
+        const float dot = (qa.x - c.v0) * (qb.x - c.v0) + (qa.y - c.v1) * (qb.y - c.v1) +
+                          (qa.z - c.v2) * (qb.z - c.v2);
+        const float g = sqrtf(sa * sb);
+        if (dot < (c.c - e) * g) return false;
+        if (sa <= ka * (1.0f - e) && sb <= kb * (1.0f - e) && dot > (c.c + e) * g) return true;
+      }
+    }
+  }
+  const long long ix = (long long)dx, iy = (long long)dy, iz = (long long)dz;
+  const long long dx2 = ix * ix + iy * iy + iz * iz;
+  return dx2 < c.T && link6(dx2, qa, qb, c.L);
+}
+
+__device__ __forceinline__ float4 pos_f32(int4 p) {
+  return make_float4((float)p.x, (float)p.y, (float)p.z, 0.0f);
+}
+
+// Pairs inside every tile (the uniting modes): each lane tests its member against the
+// later ones of the tile, ballots make the links symmetric, and the components are
+// labelled by their smallest lane with shuffles: nothing else touches the tile's members
+// yet, so the sets are written without atomics. trep[tile] = the first member that can
+// unite if all such members are now in one set, kRepNone if the tile holds none, kRepMixed
+// otherwise: k_link6 skips a pair of one-set tiles that already share a root in the box
+// test, 32 tiles at a time. In a halo's core nearly every tile pair within reach is such a
+// pair (field 6DFOF of a 200^3 box, 3.2M members: @SELF@).
+constexpr int kRepNone = -1, kRepMixed = -2;
+
+template <int MODE>
+__global__ void __launch_bounds__(128) k_link6_self(
+    const uint32_t *__restrict__ toff, const uint32_t *__restrict__ coff,
+    const uint32_t *__restrict__ thalo, int64_t t0, int64_t t1, const int4 *__restrict__ cu,
+    const float4 *__restrict__ cv, const double *__restrict__ hp, double vr2, double cos2,
+    int use_lv, int use_vt, int *__restrict__ parent, int *__restrict__ trep, GrowArgs G) {
+  __shared__ float4 s_u[4][32], s_v[4][32];
+  __shared__ float s_s[4][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned FULL = 0xffffffffu;
+  const int64_t ti = t0 + (int64_t)blockIdx.x * 4 + w;  // tiles [t0, t1)
+  if (ti >= t1) return;
+  const uint32_t h = thalo[ti];
+  const LinkC c = link_consts(hp + (int64_t)h * VR_HALO_COLS, MODE == kLink ? 1.0 : G.gx, vr2, cos2,
+                              use_lv, use_vt);
+  const uint32_t ia = coff[h] + 32u * ((uint32_t)ti - toff[h]);
+  const int na = (int)min(32u, coff[h + 1] - ia);
+  const bool va = lane < na;
+  float4 fa = pos_f32(cu[va ? ia + lane : ia]);
+  const float4 qa = cv[va ? ia + lane : ia];
+  const bool mine = va && (MODE == kLink || G.tag[ia + lane] < 0);  // may unite
+  float sa = 0.0f, ra = 0.0f;
+  if (use_vt) frame_len(c, qa, sa, ra);
+  fa.w = ra;
+  s_u[w][lane] = fa;
+  s_v[w][lane] = qa;
+  s_s[w][lane] = sa;
+  const unsigned who = __ballot_sync(FULL, mine);
+  __syncwarp();
+  unsigned adj = 0;
+  for (int k = 1; k < na; ++k) {
+    bool link = false;
+    if (mine && lane < k && ((who >> k) & 1u)) {
+      const float4 fb = s_u[w][k];
+      link = pair_link(c, fa, qa, sa, ra, fb, s_v[w][k], s_s[w][k], fb.w);
+    }
+    const unsigned b = __ballot_sync(FULL, link);
+    if (link) adj |= 1u << k;
+    if (lane == k) adj |= b;
+  }
+  int lab = lane;
+  for (;;) {
+    int next = lab;
+    for (int k = 0; k < na; ++k) {
+      const int lk = __shfl_sync(FULL, lab, k);
+      if ((adj >> k) & 1u) next = min(next, lk);
+    }
+    const bool same = next == lab;
+    lab = next;
+    if (__all_sync(FULL, same)) break;
+  }
+  if (va) parent[ia + lane] = (int)(ia + lab);
+  const int first = who ? __ffs(who) - 1 : 0;
+  const int l0 = __shfl_sync(FULL, lab, first);
+  const bool one = __all_sync(FULL, !mine || lab == l0);
+  if (lane == 0) trep[ti] = who == 0 ? kRepNone : (one ? (int)ia + first : kRepMixed);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(256) k_link6(const uint32_t *__restrict__ toff,
                                                const uint32_t *__restrict__ coff,
@@ -194,9 +344,11 @@ __global__ void __launch_bounds__(256) k_link6(const uint32_t *__restrict__ toff
                                                const int4 *__restrict__ tmax,
                                                const double *__restrict__ hp, double vr2,
                                                double cos2, int use_lv, int use_vt, int *parent,
-                                               GrowArgs G) {
-  __shared__ int4 s_u[8][32];  // one row per warp (up to 8 warps per block)
+                                               const int *__restrict__ trep, GrowArgs G) {
+  constexpr bool kUnion = MODE == kLink || MODE == kUntagged;
+  __shared__ float4 s_u[8][32];  // one row per warp (up to 8 warps per block)
   __shared__ float4 s_v[8][32];
+  __shared__ float s_s[8][32];
   __shared__ int s_r[8][32];
   __shared__ int s_x[8][32];
   __shared__ int s_y[8][32];
@@ -204,106 +356,109 @@ __global__ void __launch_bounds__(256) k_link6(const uint32_t *__restrict__ toff
   const unsigned FULL = 0xffffffffu;
   const int64_t ti = t0 + (int64_t)blockIdx.x * (blockDim.x / 32) + w;  // tiles [t0, t1)
   if (ti >= t1) return;
+  const int arep = kUnion ? trep[ti] : kRepMixed;
+  if (arep == kRepNone) return;
   const uint32_t h = thalo[ti];
-  const double *row = hp + (int64_t)h * VR_HALO_COLS;
-  Link6 L;
-  L.lx2 = row[VR_H_LX2];
-  L.lv2 = row[VR_H_LV2];
-  L.vf0 = row[VR_H_VFX];
-  L.vf1 = row[VR_H_VFY];
-  L.vf2 = row[VR_H_VFZ];
-  if (MODE != kLink) L.lx2 = __dmul_rn(__dmul_rn(L.lx2, G.gx), G.gx);
-  L.vr2 = vr2;
-  L.cos2 = cos2;
-  L.use_lv = use_lv;
-  L.use_vt = use_vt;
-  const bool fast = L.lx2 > 1e-30 && L.lx2 < 1e30 && (!use_lv || (L.lv2 > 1e-30 && L.lv2 < 1e30));
-  const float ilx2 = fast ? (float)(1.0 / L.lx2) : 0.0f;
-  const float ilv2 = fast && use_lv ? (float)(1.0 / L.lv2) : 0.0f;
+  const LinkC c = link_consts(hp + (int64_t)h * VR_HALO_COLS, MODE == kLink ? 1.0 : G.gx, vr2, cos2,
+                              use_lv, use_vt);
   const uint32_t c0h = coff[h], c1h = coff[h + 1], th0 = toff[h], th1 = toff[h + 1];
   const uint32_t ia = c0h + 32u * ((uint32_t)ti - th0);
   const uint32_t na = min(32u, c1h - ia);
   const bool va = (uint32_t)lane < na;
-  const int4 pa = cu[va ? ia + lane : ia];
+  const float4 fa = pos_f32(cu[va ? ia + lane : ia]);
   const float4 qa = cv[va ? ia + lane : ia];
+  float sa = 0.0f, ra = 0.0f;
+  if (use_vt) frame_len(c, qa, sa, ra);
   const int4 alo = tmin[ti], ahi = tmax[ti];
   const int xa = MODE == kLink || !va ? -1 : (MODE == kCross ? G.grown[ia + lane] : G.tag[ia + lane]);
   const int ya = MODE == kToGroup && va ? G.croot[ia + lane] : -1;
-  // the spatial term alone must be < 1: dx2 < lx2
-  for (uint32_t base = (uint32_t)ti; base < th1; base += 32) {
+  // lanes whose member this mode has a use for
+  const bool mine = va && (MODE == kUntagged ? xa < 0 : (MODE == kCross ? xa >= 0 : true));
+  // the spatial term alone must be < 1: dx2 < lx2. The counting modes take the pairs inside
+  // the tile here too (the uniting ones: k_link6_self)
+  for (uint32_t base = (uint32_t)ti + (kUnion ? 1u : 0u); base < th1; base += 32) {
     const uint32_t tj = base + lane;
     bool hit = false;
+    int brep = kRepMixed;
     if (tj < th1) {
       const int4 blo = tmin[tj], bhi = tmax[tj];
       const long long gx = gap1(alo.x, ahi.x, blo.x, bhi.x), gy = gap1(alo.y, ahi.y, blo.y, bhi.y),
                       gz = gap1(alo.z, ahi.z, blo.z, bhi.z);
-      hit = (double)(gx * gx + gy * gy + gz * gz) < L.lx2;
+      hit = gx * gx + gy * gy + gz * gz < c.T;
+      if (kUnion && hit) {
+        brep = trep[tj];
+        hit = brep != kRepNone;
+      }
+    }
+    if (kUnion && arep >= 0 && __any_sync(FULL, hit && brep >= 0)) {
+      const int r0 = uf_find(parent, arep);
+      if (hit && brep >= 0) hit = uf_find(parent, brep) != r0;
     }
     unsigned hm = __ballot_sync(FULL, hit);
     while (hm) {
-      const uint32_t tb = base + (uint32_t)(__ffs(hm) - 1);
+      const int src = __ffs(hm) - 1;
+      const uint32_t tb = base + (uint32_t)src;
       hm &= hm - 1;
       const uint32_t ib = c0h + 32u * (tb - th0);
       const uint32_t nbb = min(32u, c1h - ib);
+      const bool vb = (uint32_t)lane < nbb;
+      // two one-set tiles: one link settles the pair
+      const bool once = kUnion && arep >= 0 && __shfl_sync(FULL, brep, src) >= 0;
       __syncwarp();
       // current roots of both tiles' members: a tile pair whose members all share one set
       // has nothing left to link (sets only ever merge, so an equal pair of roots, even
       // stale ones, proves the two members connected)
-      constexpr bool kUnion = MODE == kLink || MODE == kUntagged;
-      const int ra = kUnion && va ? uf_find(parent, (int)(ia + lane)) : -1;
-      const int rb = kUnion && (uint32_t)lane < nbb ? uf_find(parent, (int)(ib + lane)) : -1;
-      if ((uint32_t)lane < nbb) {
-        s_u[w][lane] = cu[ib + lane];
-        s_v[w][lane] = cv[ib + lane];
-        s_r[w][lane] = rb;
-        if (MODE != kLink) s_x[w][lane] = MODE == kCross ? G.grown[ib + lane] : G.tag[ib + lane];
+      const int xb = MODE == kLink || !vb ? -1 : (MODE == kCross ? G.grown[ib + lane] : G.tag[ib + lane]);
+      const bool ours = vb && (MODE == kUntagged ? xb < 0 : (MODE == kCross ? xb >= 0 : true));
+      const int ra0 = kUnion && mine ? uf_find(parent, (int)(ia + lane)) : -1;
+      const int rb0 = kUnion && ours ? uf_find(parent, (int)(ib + lane)) : -1;
+      if (kUnion) {
+        const unsigned who = __ballot_sync(FULL, mine);
+        const int r0 = __shfl_sync(FULL, ra0, __ffs(who) - 1);
+        if (__all_sync(FULL, (!mine || ra0 == r0) && (!ours || rb0 == r0))) continue;
+      }
+      if (vb) {
+        float4 f = pos_f32(cu[ib + lane]);
+        const float4 q = cv[ib + lane];
+        if (use_vt) frame_len(c, q, s_s[w][lane], f.w);
+        s_u[w][lane] = f;
+        s_v[w][lane] = q;
+        s_r[w][lane] = rb0;
+        if (MODE != kLink) s_x[w][lane] = xb;
         if (MODE == kToGroup) s_y[w][lane] = G.croot[ib + lane];
       }
-      if (kUnion) {
-        const int r0 = __shfl_sync(FULL, ra, 0);
-        if (__all_sync(FULL, (!va || ra == r0) && ((uint32_t)lane >= nbb || rb == r0))) continue;
-      }
+      unsigned use = __ballot_sync(FULL, ours);
       __syncwarp();
-      if (!va) continue;
-      int rk = ra;  // a member of this lane's set, for the connected-pair skip below
-      for (uint32_t k = tb == (uint32_t)ti ? (uint32_t)lane + 1 : 0; k < nbb; ++k) {
+      int rk = ra0;  // a member of this lane's set, for the connected-pair skip below
+      bool done = false;
+      for (int step = 0; use; ++step) {
+        const uint32_t k = (uint32_t)__ffs(use) - 1u;
+        use &= use - 1u;
+        bool go = mine && !(tb == (uint32_t)ti && k <= (uint32_t)lane);
         // pairs this mode has no use for, before any arithmetic
-        if (MODE == kUntagged && (xa >= 0 || s_x[w][k] >= 0)) continue;
-        if (MODE == kToGroup && (xa < 0) == (s_x[w][k] < 0)) continue;
-        if (MODE == kCross && (xa < 0 || s_x[w][k] < 0 || xa == s_x[w][k])) continue;
-        const int4 p = s_u[w][k];
-        const float4 q = s_v[w][k];
-        const long long dx = (long long)pa.x - p.x, dy = (long long)pa.y - p.y,
-                        dz = (long long)pa.z - p.z;
-        const long long dx2 = dx * dx + dy * dy + dz * dz;
-        // exact pre-test: dx2 >= lx2 gives dx2 / lx2 >= 1 after rounding, so q >= 1
-        if ((double)dx2 >= L.lx2) continue;
-        bool link;
-        if (fast) {
-          float qf = (float)dx2 * ilx2;
-          if (use_lv) {
-            const float d0 = qa.x - q.x, d1 = qa.y - q.y, d2 = qa.z - q.z;
-            qf += ((d0 * d0 + d1 * d1) + d2 * d2) * ilv2;
-          }
-          if (qf >= 1.0f + 1e-5f) continue;  // also +inf; NaN falls through to FP64
-          link = (qf <= 1.0f - 1e-5f && !use_vt) ? true : link6(dx2, qa, q, L);
-        } else {
-          link = link6(dx2, qa, q, L);
+        if (kUnion) go = go && s_r[w][k] != rk;
+        if (MODE == kToGroup) go = go && (xa < 0) != (s_x[w][k] < 0);
+        if (MODE == kCross) go = go && xa != s_x[w][k];
+        bool link = false;
+        if (go) {
+          const float4 fb = s_u[w][k];
+          link = pair_link(c, fa, qa, sa, ra, fb, s_v[w][k], use_vt ? s_s[w][k] : 0.0f, fb.w);
         }
-        if (!link) continue;
-        if (kUnion) {
-          if (s_r[w][k] != rk) {
+        if (link) {
+          done = true;
+          if (kUnion) {
             uf_unite(parent, (int)(ia + lane), (int)(ib + k));
             rk = min(rk, s_r[w][k]);  // now in this lane's set
+          } else if (MODE == kToGroup) {
+            const u64 cp = (u64)(uint32_t)(xa < 0 ? ya : s_y[w][k]);
+            const u64 g = (u64)(uint32_t)(xa < 0 ? s_x[w][k] : xa);
+            hash_add(G, (cp << 32) | g);
+          } else {
+            const int b = s_x[w][k];
+            hash_add(G, ((u64)(uint32_t)min(xa, b) << 32) | (u64)(uint32_t)max(xa, b));
           }
-        } else if (MODE == kToGroup) {
-          const u64 c = (u64)(uint32_t)(xa < 0 ? ya : s_y[w][k]);
-          const u64 g = (u64)(uint32_t)(xa < 0 ? s_x[w][k] : xa);
-          hash_add(G, (c << 32) | g);
-        } else {
-          const int b = s_x[w][k];
-          hash_add(G, ((u64)(uint32_t)min(xa, b) << 32) | (u64)(uint32_t)max(xa, b));
         }
+        if (once && (step & 3) == 3 && __any_sync(FULL, done)) break;
       }
     }
   }
@@ -330,13 +485,22 @@ __global__ void k_cand_init(int64_t nc, int *__restrict__ parent, int *__restric
   size[c] = 0;
 }
 
+// Root of every candidate, the minimum particle index and the size per root. Neighbours
+// along the curve mostly share a root: a warp's lanes of one root combine first, and one of
+// them updates it.
 __global__ void k_cand_roots(int *parent, const float4 *__restrict__ cv, int64_t nc,
                              int *__restrict__ minidx, int *__restrict__ size) {
-  int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nc) return;
-  int r = uf_find(parent, (int)c);
-  atomicMin(&minidx[r], __float_as_int(cv[c].w));
-  atomicAdd(&size[r], 1);
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const bool valid = c < nc;
+  const int r = valid ? uf_find(parent, (int)c) : -1 - lane;
+  const int pi = valid ? __float_as_int(cv[c].w) : 0x7fffffff;
+  const unsigned peers = __match_any_sync(0xffffffffu, r);
+  const int m = __reduce_min_sync(peers, pi);
+  if (valid && lane == __ffs(peers) - 1) {
+    atomicMin(&minidx[r], m);
+    atomicAdd(&size[r], __popc(peers));
+  }
 }
 
 __global__ void k_cand_label(int *parent, const float4 *__restrict__ cv, int64_t nc,
@@ -375,6 +539,7 @@ size_t fof6d_bytes(int64_t n, int nmin) {
   ar.take<uint32_t>(tmaxn);     // thalo
   ar.take<int4>(tmaxn);
   ar.take<int4>(tmaxn);
+  ar.take<int>(tmaxn);  // trep
   ar.take<int>(n);  // parent
   ar.take<int>(n);  // minidx
   ar.take<int>(n);  // size
@@ -407,6 +572,7 @@ struct Cands {
   uint32_t *chid;  // halo of each candidate
   uint32_t *coff, *toff, *thalo;
   int4 *tmin, *tmax;
+  int *trep;  // per tile, see k_link6_self
   int *parent, *minidx, *size;
 };
 
@@ -425,6 +591,7 @@ vr_status prep_cands(vr_ctx *ctx, const HaloSeg &g, int nmin, Arena &ar, const f
   C->thalo = ar.take<uint32_t>(tmaxn);
   C->tmin = ar.take<int4>(tmaxn);
   C->tmax = ar.take<int4>(tmaxn);
+  C->trep = ar.take<int>(tmaxn);
   C->parent = ar.take<int>(g.n);
   C->minidx = ar.take<int>(g.n);
   C->size = ar.take<int>(g.n);
@@ -456,6 +623,26 @@ vr_status prep_cands(vr_ctx *ctx, const HaloSeg &g, int nmin, Arena &ar, const f
   k_cand_init<<<grid_for(C->nc, T), T, 0, s>>>(C->nc, C->parent, C->minidx, C->size);
   VR_LAUNCHED(ctx, "k_cand_init");
   return VR_OK;
+}
+
+// Launches of the linker over tiles [t0, t1) (counted like every launch).
+template <int MODE>
+cudaError_t link_self(const Cands &C, int64_t t0, int64_t t1, const double *hp, double vr2, double cos2,
+                      int use_lv, int use_vt, const GrowArgs &G, cudaStream_t s) {
+  k_link6_self<MODE><<<grid_for(t1 - t0, 4), 128, 0, s>>>(C.toff, C.coff, C.thalo, t0, t1, C.cu, C.cv, hp,
+                                                          vr2, cos2, use_lv, use_vt, C.parent, C.trep, G);
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <int MODE>
+cudaError_t link_tiles(const Cands &C, int64_t t0, int64_t t1, int warps, const double *hp, double vr2,
+                       double cos2, int use_lv, int use_vt, const GrowArgs &G, cudaStream_t s) {
+  k_link6<MODE><<<grid_for(t1 - t0, warps), 32 * warps, 0, s>>>(
+      C.toff, C.coff, C.thalo, t0, t1, C.cu, C.cv, C.tmin, C.tmax, hp, vr2, cos2, use_lv, use_vt,
+      C.parent, C.trep, G);
+  count_launch();
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------- two-stage linking kernels
@@ -677,19 +864,16 @@ vr_status run_fof6d(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &ar
     VR_CUDA(ctx, cudaStreamSynchronize(s));
     for (int64_t h = 0; h < H; ++h) {
       if (th[h + 1] == th[h]) continue;
-      k_link6<kLink><<<grid_for(th[h + 1] - th[h], 4), 128, 0, s>>>(
-          C.toff, C.coff, C.thalo, th[h], th[h + 1], C.cu, C.cv, C.tmin, C.tmax, hp, vr2, cos2,
-          p->use_lv, p->use_vr_theta, C.parent, G);
-      VR_LAUNCHED(ctx, "k_link6");
+      VR_CUDA(ctx, link_self<kLink>(C, th[h], th[h + 1], hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s));
+      VR_CUDA(ctx, link_tiles<kLink>(C, th[h], th[h + 1], 4, hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s));
     }
   } else {
     // tiles per block from the tuning state; a linker still to be tuned is run once per
     // candidate shape from fresh sets (same labels each time) and keeps the fastest
-    auto link = [&](int sh) {
-      const int w = kLWarps[sh];
-      k_link6<kLink><<<grid_for(C.ntiles, w), 32 * w, 0, s>>>(
-          C.toff, C.coff, C.thalo, 0, C.ntiles, C.cu, C.cv, C.tmin, C.tmax, hp, vr2, cos2,
-          p->use_lv, p->use_vr_theta, C.parent, G);
+    auto link = [&](int sh) -> cudaError_t {
+      const cudaError_t e = link_self<kLink>(C, 0, C.ntiles, hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s);
+      return e != cudaSuccess ? e : link_tiles<kLink>(C, 0, C.ntiles, kLWarps[sh], hp, vr2, cos2,
+                                                      p->use_lv, p->use_vr_theta, G, s);
     };
     if (lmeasure(ctx)) {
       Tuning *tn = ctx->tune;
@@ -703,8 +887,7 @@ vr_status run_fof6d(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &ar
           VR_LAUNCHED(ctx, "k_cand_init");
         }
         VR_CUDA(ctx, cudaEventRecord(e0, s));
-        link(sh);
-        VR_LAUNCHED(ctx, "k_link6");
+        VR_CUDA(ctx, link(sh));
         VR_CUDA(ctx, cudaEventRecord(e1, s));
         VR_CUDA(ctx, cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -717,8 +900,7 @@ vr_status run_fof6d(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &ar
       tn->lshape = best;
       tn->ltuned = 1;
     } else {
-      VR_TIMED(ctx, "link6", s, link(lshape_for(ctx)));
-      VR_LAUNCHED(ctx, "k_link6");
+      VR_TIMED(ctx, "link6", s, VR_CUDA(ctx, link(lshape_for(ctx))));
     }
   }
   k_cand_roots<<<grid_for(C.nc, T), T, 0, s>>>(C.parent, C.cv, C.nc, C.minidx, C.size);
@@ -759,21 +941,15 @@ vr_status run_grow(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, const vr_g
   const double vr = p->v_ratio * gp->gamma_vr, ct = cos(p->theta_op * gp->gamma_theta);
   const double vr2 = vr * vr, cos2 = ct * ct;
   GrowArgs G{gp->gamma_x, tag, croot, grown, hkey, hcnt, (u64)(cap - 1), ctx->d_status};
-  auto pass = [&](auto kernel) {
-    kernel<<<grid_for(C.ntiles, 4), 128, 0, s>>>(C.toff, C.coff, C.thalo, 0, C.ntiles, C.cu, C.cv,
-                                                 C.tmin, C.tmax, hp, vr2, cos2, p->use_lv,
-                                                 p->use_vr_theta, C.parent, G);
-  };
   // 1. components of the untagged candidates
-  pass(k_link6<kUntagged>);
-  VR_LAUNCHED(ctx, "k_link6<untagged>");
+  VR_CUDA(ctx, link_self<kUntagged>(C, 0, C.ntiles, hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s));
+  VR_CUDA(ctx, link_tiles<kUntagged>(C, 0, C.ntiles, 4, hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s));
   k_grow_roots<<<grid_for(nc, T), T, 0, s>>>(C.parent, nc, croot);
   VR_LAUNCHED(ctx, "k_grow_roots");
   // 2. links from components to groups; each component joins its most linked group
   k_hash_clear<<<grid_for(cap, T), T, 0, s>>>(hkey, hcnt, cap);
   VR_LAUNCHED(ctx, "k_hash_clear");
-  pass(k_link6<kToGroup>);
-  VR_LAUNCHED(ctx, "k_link6<to_group>");
+  VR_CUDA(ctx, link_tiles<kToGroup>(C, 0, C.ntiles, 4, hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s));
   k_grow_attach<<<grid_for(cap, T), T, 0, s>>>(hkey, hcnt, cap, best);
   VR_LAUNCHED(ctx, "k_grow_attach");
   k_grow_label<<<grid_for(nc, T), T, 0, s>>>(tag, croot, best, nc, grown);
@@ -781,8 +957,7 @@ vr_status run_grow(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, const vr_g
   // 3. links between grown groups; joins above the merge threshold
   k_hash_clear<<<grid_for(cap, T), T, 0, s>>>(hkey, hcnt, cap);
   VR_LAUNCHED(ctx, "k_hash_clear");
-  pass(k_link6<kCross>);
-  VR_LAUNCHED(ctx, "k_link6<cross>");
+  VR_CUDA(ctx, link_tiles<kCross>(C, 0, C.ntiles, 4, hp, vr2, cos2, p->use_lv, p->use_vr_theta, G, s));
   k_iota<<<grid_for(n, T), T, 0, s>>>(gpar, n);
   VR_LAUNCHED(ctx, "k_iota");
   k_grow_merge<<<grid_for(cap, T), T, 0, s>>>(hkey, hcnt, cap, n0, gp->f_merge, gpar);
@@ -860,10 +1035,10 @@ vr_status run_cores(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, const vr_
     if (st != VR_OK) return st;
     if (C.nc == 0) break;
     GrowArgs G{};
-    VR_TIMED(ctx, "core_link", s, k_link6<kLink><<<grid_for(C.ntiles, 4), 128, 0, s>>>(
-        C.toff, C.coff, C.thalo, 0, C.ntiles, C.cu, C.cv, C.tmin, C.tmax, hs, 0.0, 0.0, 1, 0,
-        C.parent, G));
-    VR_LAUNCHED(ctx, "k_link6");
+    timer_begin(ctx, "core_link", s);
+    VR_CUDA(ctx, link_self<kLink>(C, 0, C.ntiles, hs, 0.0, 0.0, 1, 0, G, s));
+    VR_CUDA(ctx, link_tiles<kLink>(C, 0, C.ntiles, 4, hs, 0.0, 0.0, 1, 0, G, s));
+    timer_end(ctx, "core_link", s);
     k_cand_roots<<<grid_for(C.nc, T), T, 0, s>>>(C.parent, C.cv, C.nc, C.minidx, C.size);
     VR_LAUNCHED(ctx, "k_cand_roots");
     k_core_best<<<grid_for(C.nc, T), T, 0, s>>>(C.parent, C.chid, C.nc, C.minidx, C.size, p->nmin,
