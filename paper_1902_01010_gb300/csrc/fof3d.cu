@@ -12,23 +12,27 @@
 //     position of the sub-cell inside it) with the library's radix sort, which makes
 //     every sub-cell, link cell and coarse cell (2^q link cells per axis) one contiguous
 //     run;
-//  3. a dense table over coarse cells gives each link-cell lookup in one load plus a
-//     short binary search; before it, one bit per link cell (the grid folded to 2^m
-//     cells per axis, 8 n bits or more, 4x4x4 cells per 64-bit word) tells most empty
-//     neighbours apart in one cached load: a clear bit means an empty link cell, a set
-//     bit (the cell, or one folded onto it, holds particles) goes on to the lookup;
-//  4. link cells are listed as runs of sub-cells; a warp takes 32 consecutive link cells,
-//     each lane screening one against the bitmap of its 13 forward neighbours. A lane
-//     whose link cell is one sub-cell links it on its own (a lookup and the sub-cell
-//     pairs per occupied neighbour); a link cell of several sub-cells is taken by the
-//     whole warp: lanes 0-12 find the 13 neighbours at once, the neighbour sub-cells are
-//     gathered in shared memory, and the (own, neighbour) and (own, own) sub-cell pairs
-//     are spread over the lanes. A pair of sub-cells with at most 4 member pairs is
-//     tested particle by particle; otherwise box distances settle most pairs (none
-//     linked / all linked), the rest are skipped when A and B are already in one
-//     component, else particles are tested until a linked pair is found. Linked
-//     sub-cells are merged by a lock-free union-find (atomicCAS hooks the larger root
-//     under the smaller; finds halve paths);
+//  3. link cells are listed in sort order (key, first sub-cell); a dense table over coarse
+//     cells gives the link cells of each, so a lookup is one load and a short binary search
+//     over link cells; before it, one bit per link cell (the grid folded to 2^m cells per
+//     axis, 8 n bits or more, 4x4x4 cells per 64-bit word) tells most empty neighbours apart
+//     in one cached load: a clear bit means an empty link cell, a set bit (the cell, or one
+//     folded onto it, holds particles) goes on to the lookup;
+//  4. three linking kernels over a lock-free union-find of sub-cells (atomicCAS hooks the
+//     larger root under the smaller; finds halve paths):
+//      - k_fof_own links the sub-cells of each link cell among themselves and marks the
+//        link cells that end as one set;
+//      - k_fof_neigh: a warp takes 32 consecutive link cells, screens their 13 forward
+//        neighbours against the bitmap, and spreads the occupied (cell, neighbour) pairs
+//        over its lanes. A pair of one-set cells that already share a root is done; a pair
+//        of few members is tested by its lane; the rest go to a list;
+//      - k_fof_heavy: one warp per listed pair of link cells, sub-cell pair by sub-cell
+//        pair, the large ones tested by all lanes together. By then most listed pairs
+//        share a root and cost two finds.
+//     Pairs of sub-cells with at most 4 member pairs are tested particle by particle;
+//     otherwise box distances settle most pairs (none linked / all linked), the rest are
+//     skipped when A and B are already in one component, else particles are tested until a
+//     linked pair is found;
 //  5. labels are the minimum original index of each component (atomicMin per root).
 // The grid is not a power of two per axis: the last sub-cell of each axis may be
 // partial, and box tests use each cell's true extent across the periodic edge.
@@ -92,33 +96,32 @@ FofGeom fof_geom(int64_t link_d2, int64_t n) {
 }
 
 struct FofBufs {
-  u64 *k0, *k1;
-  uint32_t *v0, *v1;
+  u64 *k0, *k1;        // sort keys; the spare one: scan buffer, then list of heavy pairs, then
+                       // minimum index per root
+  uint32_t *v0, *v1;   // sort values (n + 1 each): sub-cell of each particle, and (once the
+                       // positions are gathered) first sub-cell of each link cell
   int4 *posS;
-  int *parent;
-  int *minidx;
-  uint32_t *head;     // 1 at the first particle of each sub-cell, then its exclusive scan
-  uint32_t *sc_start; // first sorted index of each sub-cell
-  uint32_t *cstart, *cend;
+  int *parent;         // union-find over sub-cells
+  uint32_t *sc_start;  // first sorted index of each sub-cell
+  u64 *lckey;          // key of each link cell, kOneSet in its top bit
+  uint2 *ctab;         // link cells [x, y) of each coarse cell
   unsigned long long *occ;  // occupancy bitmap of the link cells
-  void *scratch;      // radix sort / scan scratch
+  void *scratch;       // radix sort / scan scratch, then the list's counter
 };
 
 FofBufs fof_carve(Arena &ar, int64_t n, int64_t ncoarse, int om) {
   FofBufs b;
-  b.k0 = ar.take<u64>(n + 1);  // n + 1: the spare one holds 2 n + 2 link-cell words
+  b.k0 = ar.take<u64>(n + 1);
   b.k1 = ar.take<u64>(n + 1);
-  b.v0 = ar.take<uint32_t>(n);
-  b.v1 = ar.take<uint32_t>(n);
+  b.v0 = ar.take<uint32_t>(n + 1);
+  b.v1 = ar.take<uint32_t>(n + 1);
   b.posS = ar.take<int4>(n);
   b.parent = ar.take<int>(n);
-  b.minidx = ar.take<int>(n);
-  b.head = ar.take<uint32_t>(n + 1);
   b.sc_start = ar.take<uint32_t>(n + 1);
-  b.cstart = ar.take<uint32_t>(ncoarse);
-  b.cend = ar.take<uint32_t>(ncoarse);
+  b.lckey = ar.take<u64>(n);
+  b.ctab = ar.take<uint2>(ncoarse);
   b.occ = ar.take<unsigned long long>(occ_words(om));
-  size_t a = radix_scratch_bytes<u64>(n), c = scan_scratch_bytes<uint32_t>(n + 1);
+  size_t a = radix_scratch_bytes<u64>(n), c = scan_scratch_bytes<u64>(n + 1);
   b.scratch = ar.take<char>(a > c ? a : c);
   return b;
 }
@@ -162,58 +165,63 @@ __global__ void k_fof_keys(const int32_t *__restrict__ pos, int64_t n, int S, in
 }
 
 
+// Positions in sorted order, and per particle the two start flags to be scanned together:
+// high word 1 at the first particle of a sub-cell, low word 1 at that of a link cell.
 __global__ void k_fof_prepare(const int32_t *__restrict__ pos, const u64 *__restrict__ keyS,
-                              const uint32_t *__restrict__ orig, int64_t n, int cshift,
-                              int4 *__restrict__ posS, int *__restrict__ minidx,
-                              uint32_t *__restrict__ head, uint32_t *__restrict__ cstart,
-                              uint32_t *__restrict__ cend, unsigned long long *__restrict__ occ,
-                              int om) {
+                              const uint32_t *__restrict__ orig, int64_t n,
+                              int4 *__restrict__ posS, u64 *__restrict__ flag) {
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p > n) return;
   if (p == n) {
-    head[n] = 0;
+    flag[n] = 0;
     return;
   }
   int64_t i = orig[p];
   const uint32_t m = (uint32_t)kLattice - 1u;
   posS[p] = make_int4((int)((uint32_t)pos[3 * i] & m), (int)((uint32_t)pos[3 * i + 1] & m),
                       (int)((uint32_t)pos[3 * i + 2] & m), (int)i);
-  minidx[p] = 0x7fffffff;
-  u64 k = keyS[p];
-  head[p] = (p == 0 || keyS[p - 1] != k) ? 1u : 0u;
-  if (p == 0 || (keyS[p - 1] >> 6) != (k >> 6)) {  // first particle of its link cell
+  const u64 d = p == 0 ? ~0ull : keyS[p - 1] ^ keyS[p];
+  flag[p] = d == 0 ? 0ull : ((1ull << 32) | (d >> 6 ? 1ull : 0ull));
+}
+
+// excl = the exclusive scan of the flags. Sub-cell of every particle, start of every
+// sub-cell (sc_start[nsc] = n), key and first sub-cell of every link cell (lcfirst[nlc] =
+// nsc), link cells of every coarse cell, the occupancy bitmap, and one set per sub-cell:
+// all its members are within the linking length of each other (3 (S-1)^2 < link_d2).
+__global__ void k_fof_cells(const u64 *__restrict__ keyS, const u64 *__restrict__ excl, int64_t n,
+                            int cshift, uint32_t *__restrict__ sid, uint32_t *__restrict__ sc_start,
+                            uint32_t *__restrict__ lcfirst, u64 *__restrict__ lckey,
+                            uint2 *__restrict__ ctab, unsigned long long *__restrict__ occ, int om,
+                            int *__restrict__ parent) {
+  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  const u64 e = excl[p], k = keyS[p];
+  const u64 d = p == 0 ? ~0ull : keyS[p - 1] ^ k;
+  const uint32_t sub = (uint32_t)(e >> 32) - (d ? 0u : 1u);
+  sid[p] = sub;
+  if (d) {
+    sc_start[sub] = (uint32_t)p;
+    parent[sub] = (int)sub;
+  }
+  if (d >> 6) {  // first particle of its link cell
+    const uint32_t c = (uint32_t)e;
+    lcfirst[c] = sub;
+    lckey[c] = k >> 6;
     u64 w;
     uint32_t bit;
     occ_pos(compact3(k >> 6), compact3(k >> 7), compact3(k >> 8), om, w, bit);
     atomicOr(&occ[w], 1ull << bit);
+    if (p == 0 || (d >> cshift)) {  // and of its coarse cell
+      ctab[k >> cshift].x = c;
+      if (p > 0) ctab[keyS[p - 1] >> cshift].y = c;
+    }
   }
-  u64 c = k >> cshift;
-  if (p == 0 || (keyS[p - 1] >> cshift) != c) cstart[c] = (uint32_t)p;
-  if (p == n - 1 || (keyS[p + 1] >> cshift) != c) cend[c] = (uint32_t)(p + 1);
-}
-
-// excl[p] = number of sub-cell starts before p (exclusive scan of the start flags).
-// Writes the sub-cell id of every sorted particle and the start of every sub-cell
-// (sc_start[nsc] = n).
-__global__ void k_fof_subcells(const u64 *__restrict__ keyS, const uint32_t *__restrict__ excl,
-                               int64_t n, uint32_t *__restrict__ sid,
-                               uint32_t *__restrict__ sc_start) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  bool first = (p == 0 || keyS[p - 1] != keyS[p]);
-  uint32_t id = excl[p] - (first ? 0u : 1u);
-  sid[p] = id;
-  if (first) sc_start[id] = (uint32_t)p;
-  if (p == n - 1) sc_start[id + 1] = (uint32_t)n;
-}
-
-// Every member of a sub-cell is hooked directly below the sub-cell's first particle:
-// all members are within the linking length of each other (3 (S-1)^2 < link_d2).
-__global__ void k_fof_hook(const uint32_t *__restrict__ sid, const uint32_t *__restrict__ sc_start,
-                           int64_t n, int *__restrict__ parent) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  parent[p] = (int)sc_start[sid[p]];
+  if (p == n - 1) {
+    const u64 t = excl[n];
+    sc_start[(uint32_t)(t >> 32)] = (uint32_t)n;
+    lcfirst[(uint32_t)t] = (uint32_t)(t >> 32);
+    ctab[k >> cshift].y = (uint32_t)t;
+  }
 }
 
 __device__ __forceinline__ long long d2_periodic(int4 a, int4 b) {
@@ -261,304 +269,370 @@ __device__ __forceinline__ uint32_t compact3(u64 x) {  // every third bit of x, 
 
 
 // Pairs of sub-cells with at most this many member pairs are tested particle by particle,
-// without the box tests.
-constexpr uint32_t kDirectPairs = 4;
+// without the box tests; those of more than kSerialPairs by a whole warp.
+constexpr uint32_t kDirectPairs = 4, kSerialPairs = 64;
+// Link-cell pairs of at most this many member pairs are tested by one lane of k_fof_neigh.
+constexpr uint32_t kLanePairs = 32;
+constexpr u64 kOneSet = 1ull << 63;  // lckey: the link cell's sub-cells are all in one set
 
-// Links sub-cell A = [a0, a1) with sub-cell B = [b0, b1) (sub-cell coordinates bc) if any
-// pair of their members is within the linking length.
-__device__ __forceinline__ void link_subcells(const int4 *__restrict__ posS, int *parent,
-                                              uint32_t a0, uint32_t a1, const int *alo,
-                                              const int *ahi, uint32_t b0, uint32_t b1,
-                                              uint32_t bcx, uint32_t bcy, uint32_t bcz, int S,
-                                              long long T) {
-  const uint32_t bc[3] = {bcx, bcy, bcz};
-  if ((a1 - a0) * (b1 - b0) <= kDirectPairs) {
-    for (uint32_t a = a0; a < a1; ++a) {
-      const int4 xa = posS[a];
-      for (uint32_t b = b0; b < b1; ++b) {
-        if (d2_periodic(xa, posS[b]) < T) {
-          uf_unite(parent, (int)a0, (int)b0);
-          return;
-        }
-      }
-    }
-    return;
-  }
-  long long mind = 0, maxd = 0;
-  int bl[3], bh[3];
+struct FofCells {
+  const int4 *posS;
+  const u64 *keyS;
+  const uint32_t *sc_start, *lcfirst;
+  const uint2 *ctab;
+  const unsigned long long *occ;
+  int om, S, GL, qshift;
+  long long T;
+};
+
+// Extent of sub-cell coordinates 2 l + (2-bit position of the sort key) per axis.
+__device__ __forceinline__ void sub_box(u64 key, const int *l, int S, int *lo, int *hi) {
+  cell_span(2 * l[0] + (int)((key >> 4) & 3u), S, lo[0], hi[0]);
+  cell_span(2 * l[1] + (int)((key >> 2) & 3u), S, lo[1], hi[1]);
+  cell_span(2 * l[2] + (int)(key & 3u), S, lo[2], hi[2]);
+}
+
+// Squared distance from x (inside A's box) to box B in A's frame.
+__device__ __forceinline__ long long box_gap2(int4 x, const int *bl, const int *bh) {
+  const long long gx = x.x < bl[0] ? bl[0] - x.x : (x.x > bh[0] ? x.x - bh[0] : 0);
+  const long long gy = x.y < bl[1] ? bl[1] - x.y : (x.y > bh[1] ? x.y - bh[1] : 0);
+  const long long gz = x.z < bl[2] ? bl[2] - x.z : (x.z > bh[2] ? x.z - bh[2] : 0);
+  return gx * gx + gy * gy + gz * gz;
+}
+
+// Boxes of sub-cells A and B (first particles a0, b0; link-cell coordinates la, lb), B
+// shifted into A's frame: smallest and largest squared separation of their points.
+__device__ __forceinline__ void pair_boxes(const FofCells &f, uint32_t a0, const int *la, uint32_t b0,
+                                           const int *lb, int *bl, int *bh, long long &mind,
+                                           long long &maxd) {
+  int alo[3], ahi[3], lo[3], hi[3];
+  sub_box(f.keyS[a0], la, f.S, alo, ahi);
+  sub_box(f.keyS[b0], lb, f.S, lo, hi);
+  mind = maxd = 0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    int lo, hi;
-    cell_span((int)bc[k], S, lo, hi);
     long long gp, fr;
-    int sh = axis_gap(alo[k], ahi[k], lo, hi, gp, fr);
-    bl[k] = lo + sh;
-    bh[k] = hi + sh;
+    const int sh = axis_gap(alo[k], ahi[k], lo[k], hi[k], gp, fr);
+    bl[k] = lo[k] + sh;
+    bh[k] = hi[k] + sh;
     mind += gp * gp;
     maxd += fr * fr;
   }
-  if (mind >= T) return;  // no pair can link
-  if (maxd < T) {         // every pair links
-    uf_unite(parent, (int)a0, (int)b0);
-    return;
-  }
-  if (uf_find(parent, (int)a0) == uf_find(parent, (int)b0)) return;
+}
+
+// All member pairs of sub-cells A and B, until one is within the linking length.
+__device__ __forceinline__ bool any_pair(const FofCells &f, uint32_t a0, uint32_t a1, uint32_t b0,
+                                         uint32_t b1) {
   for (uint32_t a = a0; a < a1; ++a) {
-    const int4 xa = posS[a];  // inside A's box, so no wrap in A's frame
-    long long gx = xa.x < bl[0] ? bl[0] - xa.x : (xa.x > bh[0] ? xa.x - bh[0] : 0);
-    long long gy = xa.y < bl[1] ? bl[1] - xa.y : (xa.y > bh[1] ? xa.y - bh[1] : 0);
-    long long gz = xa.z < bl[2] ? bl[2] - xa.z : (xa.z > bh[2] ? xa.z - bh[2] : 0);
-    if (gx * gx + gy * gy + gz * gz >= T) continue;
-    for (uint32_t b = b0; b < b1; ++b) {
-      if (d2_periodic(xa, posS[b]) < T) {
-        uf_unite(parent, (int)a0, (int)b0);
-        return;
+    const int4 xa = f.posS[a];
+    for (uint32_t b = b0; b < b1; ++b)
+      if (d2_periodic(xa, f.posS[b]) < f.T) return true;
+  }
+  return false;
+}
+
+// Links every sub-cell pair of link cells A = sub-cells [sa0, sa1) at la and B at lb (or
+// the pairs inside A when `own`) with a whole warp: the pairs spread over the lanes, the
+// large ones then tested by all lanes. `once`: A and B are one set each, so the first link
+// ends it.
+__device__ void link_cells_warp(const FofCells &f, int *parent, uint32_t sa0, uint32_t sa1,
+                                const int *la, uint32_t sb0, uint32_t sb1, const int *lb, bool own,
+                                bool once) {
+  const int lane = threadIdx.x & 31;
+  const unsigned FULL = 0xffffffffu;
+  const uint32_t mb = sb1 - sb0, total = (sa1 - sa0) * mb;
+  for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+    const uint32_t t = t0 + lane;
+    const uint32_t i = t / mb, j = t - i * mb;
+    const uint32_t sa = sa0 + i, sb = sb0 + j;
+    bool linked = false, large = false;
+    if (t < total && (!own || i < j)) {
+      const uint32_t a0 = f.sc_start[sa], a1 = f.sc_start[sa + 1], b0 = f.sc_start[sb],
+                     b1 = f.sc_start[sb + 1];
+      const u64 np = (u64)(a1 - a0) * (b1 - b0);
+      if (np <= kDirectPairs) {
+        linked = any_pair(f, a0, a1, b0, b1);
+        if (linked) uf_unite(parent, (int)sa, (int)sb);
+      } else {
+        int bl[3], bh[3];
+        long long mind, maxd;
+        pair_boxes(f, a0, la, b0, lb, bl, bh, mind, maxd);
+        if (mind < f.T) {
+          if (maxd < f.T) {
+            uf_unite(parent, (int)sa, (int)sb);
+            linked = true;
+          } else if (uf_find(parent, (int)sa) == uf_find(parent, (int)sb)) {
+            linked = true;
+          } else if (np <= kSerialPairs) {
+            for (uint32_t a = a0; a < a1 && !linked; ++a) {
+              const int4 xa = f.posS[a];  // inside A's box, so no wrap in A's frame
+              if (box_gap2(xa, bl, bh) >= f.T) continue;
+              for (uint32_t b = b0; b < b1 && !linked; ++b) linked = d2_periodic(xa, f.posS[b]) < f.T;
+            }
+            if (linked) uf_unite(parent, (int)sa, (int)sb);
+          } else {
+            large = true;
+          }
+        }
+      }
+    }
+    if (once && __any_sync(FULL, linked)) return;
+    unsigned lm = __ballot_sync(FULL, large);
+    while (lm) {
+      const int src = __ffs(lm) - 1;
+      lm &= lm - 1;
+      const uint32_t ua = __shfl_sync(FULL, sa, src), ub = __shfl_sync(FULL, sb, src);
+      int same = 0;
+      if (lane == 0) same = uf_find(parent, (int)ua) == uf_find(parent, (int)ub);
+      if (__shfl_sync(FULL, same, 0)) {
+        if (once) return;
+        continue;
+      }
+      const uint32_t a0 = f.sc_start[ua], a1 = f.sc_start[ua + 1], b0 = f.sc_start[ub],
+                     b1 = f.sc_start[ub + 1];
+      int bl[3], bh[3];
+      long long mind, maxd;
+      pair_boxes(f, a0, la, b0, lb, bl, bh, mind, maxd);
+      bool found = false;
+      for (uint32_t ab = a0; ab < a1 && !found; ab += 32) {  // a member of A per lane ...
+        const uint32_t a = ab + lane;
+        int4 xa = make_int4(0, 0, 0, 0);
+        bool near = false;
+        if (a < a1) {
+          xa = f.posS[a];
+          near = box_gap2(xa, bl, bh) < f.T;
+        }
+        unsigned nm = __ballot_sync(FULL, near);
+        while (nm && !found) {  // ... those within reach of B's box against B's members
+          const int s = __ffs(nm) - 1;
+          nm &= nm - 1;
+          const int4 x = make_int4(__shfl_sync(FULL, xa.x, s), __shfl_sync(FULL, xa.y, s),
+                                   __shfl_sync(FULL, xa.z, s), 0);
+          bool hit = false;
+          for (uint32_t b = b0 + lane; b < b1 && !hit; b += 32) hit = d2_periodic(x, f.posS[b]) < f.T;
+          found = __any_sync(FULL, hit);
+        }
+      }
+      if (found) {
+        if (lane == 0) uf_unite(parent, (int)ua, (int)ub);
+        if (once) return;
       }
     }
   }
 }
 
-// Sub-cell coordinates of sort key bk in link cell (lx, ly, lz): 2 l + the key's 2-bit
-// position along each axis (three comma-separated values).
-#define VR_SUB_OF(bk, lx, ly, lz)                                       \
-  2u * (uint32_t)(lx) + (uint32_t)(((bk) >> 4) & 3u),                   \
-      2u * (uint32_t)(ly) + (uint32_t)(((bk) >> 2) & 3u),               \
-      2u * (uint32_t)(lz) + (uint32_t)((bk) & 3u)
-
-// Link cells as runs of sub-cells: flag[A] = 1 at the first sub-cell A of each link cell
-// (entries [0, n]; zero from nsc on), scanned in place into link-cell ids.
-__global__ void k_fof_lcflags(const u64 *__restrict__ keyS, const uint32_t *__restrict__ sc_start,
-                              const uint32_t *__restrict__ nsc_ptr, int64_t n,
-                              uint32_t *__restrict__ flag) {
-  const int64_t A = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (A > n) return;
-  const int64_t nsc = *nsc_ptr;
-  uint32_t f = 0;
-  if (A < nsc)
-    f = (A == 0 || (keyS[sc_start[A - 1]] >> 6) != (keyS[sc_start[A]] >> 6)) ? 1u : 0u;
-  flag[A] = f;
-}
-
-// After the scan (lcf[A] = link cell of a first sub-cell A, lcf[n] = number of link
-// cells): lcfirst[c] = first sub-cell of link cell c, lcfirst[nlc] = nsc.
-__global__ void k_fof_lcfirst(const u64 *__restrict__ keyS, const uint32_t *__restrict__ sc_start,
-                              const uint32_t *__restrict__ nsc_ptr, int64_t n,
-                              const uint32_t *__restrict__ lcf, uint32_t *__restrict__ lcfirst) {
-  const int64_t A = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (A > n) return;
-  const int64_t nsc = *nsc_ptr;
-  if (A > nsc) return;
-  if (A == nsc) {
-    lcfirst[lcf[A]] = (uint32_t)nsc;
-    return;
+// Pairs of sub-cells of one link cell; lane l of a warp takes link cell c0 + l, the cells
+// of more than kLanePairs member pairs are taken by the whole warp.
+constexpr int kLW = 4;  // warps per block of the link kernels
+__global__ void __launch_bounds__(32 * kLW) k_fof_own(FofCells f, const u64 *__restrict__ excl_n,
+                                                      u64 *__restrict__ lckey, int *parent) {
+  const int lane = threadIdx.x & 31;
+  const unsigned FULL = 0xffffffffu;
+  const int64_t nlc = (uint32_t)*excl_n;
+  for (int64_t c0 = ((int64_t)blockIdx.x * kLW + (threadIdx.x >> 5)) * 32; c0 < nlc;
+       c0 += (int64_t)gridDim.x * kLW * 32) {
+    uint32_t s0 = 0, s1 = 0;
+    bool one = false, many = false;
+    if (c0 + lane < nlc) {
+      s0 = f.lcfirst[c0 + lane];
+      s1 = f.lcfirst[c0 + lane + 1];
+      one = s1 - s0 == 1;
+      if (!one) {
+        const u64 np = f.sc_start[s1] - f.sc_start[s0];
+        many = np * np > 2 * kLanePairs;
+        if (!many) {
+          for (uint32_t i = s0; i < s1; ++i)
+            for (uint32_t j = i + 1; j < s1; ++j)
+              if (any_pair(f, f.sc_start[i], f.sc_start[i + 1], f.sc_start[j], f.sc_start[j + 1]))
+                uf_unite(parent, (int)i, (int)j);
+        }
+      }
+    }
+    unsigned mm = __ballot_sync(FULL, many);
+    while (mm) {
+      const int src = __ffs(mm) - 1;
+      mm &= mm - 1;
+      const uint32_t a = __shfl_sync(FULL, s0, src), b = __shfl_sync(FULL, s1, src);
+      const u64 k = lckey[c0 + src];
+      const int l[3] = {(int)compact3(k), (int)compact3(k >> 1), (int)compact3(k >> 2)};
+      link_cells_warp(f, parent, a, b, l, a, b, l, true, false);
+      __syncwarp();
+    }
+    if (s1 - s0 > 1) {  // one set: every sub-cell has the first one's root
+      const int r = uf_find(parent, (int)s0);
+      one = true;
+      for (uint32_t i = s0 + 1; i < s1 && one; ++i) one = uf_find(parent, (int)i) == r;
+    }
+    if (one) lckey[c0 + lane] |= kOneSet;
   }
-  if (A == 0 || (keyS[sc_start[A - 1]] >> 6) != (keyS[sc_start[A]] >> 6))
-    lcfirst[lcf[A]] = (uint32_t)A;
 }
 
-constexpr int kLW = 8;       // warps per block of the link-cell kernel
-constexpr int kLCap = 128;   // neighbour sub-cells a warp holds per round
-constexpr int kLMaxSub = 64; // sub-cells of one link cell (4 x 4 x 4 at most)
-
-__device__ __forceinline__ u64 pack_sub(uint32_t x, uint32_t y, uint32_t z) {
-  return (u64)x | ((u64)y << 21) | ((u64)z << 42);
+// Link cell with key `key`, or kEmpty.
+__device__ __forceinline__ uint32_t find_cell(const FofCells &f, const u64 *__restrict__ lckey, u64 key) {
+  const uint2 r = __ldg(&f.ctab[key >> f.qshift]);
+  if (r.x == kEmpty) return kEmpty;
+  uint32_t lo = r.x, hi = r.y;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if ((__ldg(&lckey[mid]) & ~kOneSet) < key) lo = mid + 1; else hi = mid;
+  }
+  return lo < r.y && (__ldg(&lckey[lo]) & ~kOneSet) == key ? lo : kEmpty;
 }
 
-// Sub-cell pair (A, B) from packed sub-cell coordinates.
-__device__ __forceinline__ void link_pair(const int4 *__restrict__ posS, int *parent, uint32_t a0,
-                                          uint32_t a1, u64 ac, uint32_t b0, uint32_t b1, u64 bc,
-                                          int S, long long T) {
-  const u64 M = (1ull << 21) - 1ull;
-  int alo[3], ahi[3];
+__device__ __forceinline__ void fwd_cell(const int *l, int q, int GL, int *o) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) cell_span((int)((ac >> (21 * k)) & M), S, alo[k], ahi[k]);
-  link_subcells(posS, parent, a0, a1, alo, ahi, b0, b1, (uint32_t)(bc & M),
-                (uint32_t)((bc >> 21) & M), (uint32_t)(bc >> 42), S, T);
+  for (int a = 0; a < 3; ++a) {
+    const int x = l[a] + c_fwd[q][a];
+    o[a] = x < 0 ? x + GL : (x >= GL ? x - GL : x);
+  }
 }
 
-// Persistent grid; each warp takes 32 consecutive link cells (sort order) at a time. Lane l
-// screens link cell c0 + l against the occupancy bitmap of its 13 forward neighbours; a
-// single-sub-cell link cell with occupied neighbours is linked by its lane alone; a link
-// cell of several sub-cells is linked by the whole warp: the pairs of its own sub-cells,
-// then, with lanes 0-12 each finding one forward link cell, every (own sub-cell,
-// neighbour sub-cell) pair, the pairs spread over the lanes. Neighbour sub-cells are
-// gathered kLCap at a time.
-__global__ void __launch_bounds__(32 * kLW, 5) k_fof_link_w(
-    const int4 *__restrict__ posS, const u64 *__restrict__ keyS, const uint32_t *__restrict__ sid,
-    const uint32_t *__restrict__ sc_start, const uint32_t *__restrict__ lcf,
-    const uint32_t *__restrict__ lcfirst, const uint32_t *__restrict__ cstart,
-    const uint32_t *__restrict__ cend, const unsigned long long *__restrict__ occ, int om,
-    int *parent, int64_t n, int S, int GL, int qshift, long long T) {
-  __shared__ uint32_t s_b0[kLW][kLCap], s_b1[kLW][kLCap];
-  __shared__ u64 s_bc[kLW][kLCap];
-  __shared__ uint32_t s_a0[kLW][kLMaxSub + 1];
-  __shared__ u64 s_ac[kLW][kLMaxSub];
-  __shared__ int s_cnt[kLW];
+// Pairs of adjacent link cells, as described at the top. Each warp takes 32 consecutive
+// link cells at a time.
+__global__ void __launch_bounds__(32 * kLW) k_fof_neigh(FofCells f, const u64 *__restrict__ excl_n,
+                                                        const u64 *__restrict__ lckey, int *parent,
+                                                        uint2 *__restrict__ heavy, uint32_t cap,
+                                                        uint32_t *__restrict__ nheavy) {
+  __shared__ uint16_t s_task[kLW][32 * 13];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned FULL = 0xffffffffu;
-  const int64_t nlc = lcf[n];
+  const int64_t nlc = (uint32_t)*excl_n;
   for (int64_t c0 = ((int64_t)blockIdx.x * kLW + w) * 32; c0 < nlc; c0 += (int64_t)gridDim.x * kLW * 32) {
-    // lane l screens link cell c0 + l: one sub-cell and no forward neighbour in the
-    // occupancy bitmap means nothing to link
-    int my_m = 0, mfx = 0, mfy = 0, mfz = 0;
-    uint32_t my_s0 = 0, my_bits = 0;
+    uint32_t bits = 0;
     if (c0 + lane < nlc) {
-      my_s0 = lcfirst[c0 + lane];
-      my_m = (int)(lcfirst[c0 + lane + 1] - my_s0);
-      const u64 k = keyS[sc_start[my_s0]] >> 6;
-      mfx = (int)compact3(k);
-      mfy = (int)compact3(k >> 1);
-      mfz = (int)compact3(k >> 2);
-#pragma unroll 1
+      const u64 k = lckey[c0 + lane];
+      const int l[3] = {(int)compact3(k), (int)compact3(k >> 1), (int)compact3(k >> 2)};
+#pragma unroll
       for (int q = 0; q < 13; ++q) {
-        int x = mfx + c_fwd[q][0], y = mfy + c_fwd[q][1], z = mfz + c_fwd[q][2];
-        x = x < 0 ? x + GL : (x >= GL ? x - GL : x);
-        y = y < 0 ? y + GL : (y >= GL ? y - GL : y);
-        z = z < 0 ? z + GL : (z >= GL ? z - GL : z);
+        int o[3];
+        fwd_cell(l, q, f.GL, o);
         u64 ow;
         uint32_t ob;
-        occ_pos((uint32_t)x, (uint32_t)y, (uint32_t)z, om, ow, ob);
-        if ((__ldg(&occ[ow]) >> ob) & 1ull) my_bits |= 1u << q;
+        occ_pos((uint32_t)o[0], (uint32_t)o[1], (uint32_t)o[2], f.om, ow, ob);
+        bits |= (uint32_t)((__ldg(&f.occ[ow]) >> ob) & 1ull) << q;
       }
     }
-    if (my_m == 1 && my_bits != 0) {  // a single sub-cell: this lane links it on its own
-      const uint32_t a0 = sc_start[my_s0], a1 = sc_start[my_s0 + 1];
-      const u64 ak = keyS[a0];
-      int alo[3], ahi[3];
-      cell_span((int)(2u * (uint32_t)mfx + (uint32_t)((ak >> 4) & 3u)), S, alo[0], ahi[0]);
-      cell_span((int)(2u * (uint32_t)mfy + (uint32_t)((ak >> 2) & 3u)), S, alo[1], ahi[1]);
-      cell_span((int)(2u * (uint32_t)mfz + (uint32_t)(ak & 3u)), S, alo[2], ahi[2]);
-#pragma unroll 1
-      for (int q = 0; q < 13; ++q) {
-        if (!((my_bits >> q) & 1u)) continue;
-        int x = mfx + c_fwd[q][0], y = mfy + c_fwd[q][1], z = mfz + c_fwd[q][2];
-        x = x < 0 ? x + GL : (x >= GL ? x - GL : x);
-        y = y < 0 ? y + GL : (y >= GL ? y - GL : y);
-        z = z < 0 ? z + GL : (z >= GL ? z - GL : z);
-        const u64 key = morton3((uint32_t)x, (uint32_t)y, (uint32_t)z);
-        const u64 c = key >> qshift;
-        uint32_t lo = __ldg(&cstart[c]);
-        if (lo == kEmpty) continue;
-        uint32_t hi = __ldg(&cend[c]);
-        while (lo < hi) {
-          const uint32_t mid = (lo + hi) >> 1;
-          if ((keyS[mid] >> 6) < key) lo = mid + 1; else hi = mid;
-        }
-        for (uint32_t j = lo; j < (uint32_t)n;) {
-          const u64 bk = keyS[j];
-          if ((bk >> 6) != key) break;
-          const uint32_t j1 = sc_start[sid[j] + 1];
-          link_subcells(posS, parent, a0, a1, alo, ahi, j, j1, VR_SUB_OF(bk, x, y, z), S, T);
-          j = j1;
-        }
-      }
-      my_bits = 0;
+    // the occupied (cell, neighbour) pairs of the 32 cells, one after the other
+    const int mine = __popc(bits);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += y;
     }
-    unsigned todo = __ballot_sync(FULL, my_m > 1 || my_bits != 0);
-    while (todo) {
-    const int src = __ffs(todo) - 1;
-    todo &= todo - 1;
-    const uint32_t s0 = __shfl_sync(FULL, my_s0, src);
-    const int m = __shfl_sync(FULL, my_m, src);
-    const int fx = __shfl_sync(FULL, mfx, src), fy = __shfl_sync(FULL, mfy, src),
-              fz = __shfl_sync(FULL, mfz, src);
-    const uint32_t bits = __shfl_sync(FULL, my_bits, src);
-    for (int i = lane; i <= m; i += 32) {  // sub-cell starts (and the end of the last)
-      const uint32_t p0 = sc_start[s0 + i];
-      s_a0[w][i] = p0;
-      if (i < m) {
-        const u64 k = keyS[p0];
-        s_ac[w][i] = pack_sub(VR_SUB_OF(k, fx, fy, fz));
-      }
-    }
+    const int ntask = __shfl_sync(FULL, incl, 31);
+    for (int at = incl - mine; bits; bits &= bits - 1) s_task[w][at++] = (uint16_t)(lane * 16 + __ffs(bits) - 1);
     __syncwarp();
-    for (int t = lane; t < m * m; t += 32) {  // own sub-cells, i < j
-      const int i = t / m, j = t - i * m;
-      if (j <= i) continue;
-      link_pair(posS, parent, s_a0[w][i], s_a0[w][i + 1], s_ac[w][i], s_a0[w][j], s_a0[w][j + 1],
-                s_ac[w][j], S, T);
-    }
-    uint32_t cur = (uint32_t)n;  // lane k < 13: next particle of forward link cell k
-    u64 nkey = 0;
-    int nx = 0, ny = 0, nz = 0;
-    if (lane < 13 && ((bits >> lane) & 1u)) {
-      nx = fx + c_fwd[lane][0];
-      ny = fy + c_fwd[lane][1];
-      nz = fz + c_fwd[lane][2];
-      nx = nx < 0 ? nx + GL : (nx >= GL ? nx - GL : nx);
-      ny = ny < 0 ? ny + GL : (ny >= GL ? ny - GL : ny);
-      nz = nz < 0 ? nz + GL : (nz >= GL ? nz - GL : nz);
-      {
-        nkey = morton3((uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
-        const u64 c = nkey >> qshift;
-        uint32_t lo = __ldg(&cstart[c]);
-        if (lo != kEmpty) {
-          uint32_t hi = __ldg(&cend[c]);
-          while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if ((keyS[mid] >> 6) < nkey) lo = mid + 1; else hi = mid;
+    for (int t0 = 0; t0 < ntask; t0 += 32) {
+      const int t = t0 + lane;
+      uint32_t ca = 0, cb = kEmpty;
+      bool list = false;
+      if (t < ntask) {
+        const int task = s_task[w][t];
+        ca = (uint32_t)c0 + (uint32_t)(task >> 4);
+        const u64 ka = lckey[ca];
+        const int l[3] = {(int)compact3(ka), (int)compact3(ka >> 1), (int)compact3(ka >> 2)};
+        int o[3];
+        fwd_cell(l, task & 15, f.GL, o);
+        cb = find_cell(f, lckey, morton3((uint32_t)o[0], (uint32_t)o[1], (uint32_t)o[2]));
+        if (cb != kEmpty) {
+          const bool once = (ka & __ldg(&lckey[cb]) & kOneSet) != 0;
+          const uint32_t sa0 = f.lcfirst[ca], sa1 = f.lcfirst[ca + 1], sb0 = f.lcfirst[cb],
+                         sb1 = f.lcfirst[cb + 1];
+          const uint32_t a0 = f.sc_start[sa0], a1 = f.sc_start[sa1], b0 = f.sc_start[sb0],
+                         b1 = f.sc_start[sb1];
+          if ((a1 - a0) == 1 && (b1 - b0) == 1) {
+            if (d2_periodic(f.posS[a0], f.posS[b0]) < f.T) uf_unite(parent, (int)sa0, (int)sb0);
+          } else if (!(once && uf_find(parent, (int)sa0) == uf_find(parent, (int)sb0))) {
+            if ((u64)(a1 - a0) * (b1 - b0) <= kLanePairs) {
+              bool done = false;
+              for (uint32_t i = sa0; i < sa1 && !done; ++i)
+                for (uint32_t j = sb0; j < sb1 && !done; ++j)
+                  if (any_pair(f, f.sc_start[i], f.sc_start[i + 1], f.sc_start[j], f.sc_start[j + 1])) {
+                    uf_unite(parent, (int)i, (int)j);
+                    done = once;
+                  }
+            } else {
+              list = true;
+            }
           }
-          cur = lo;
+        }
+      }
+      const unsigned lm = __ballot_sync(FULL, list);
+      if (lm) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(nheavy, (uint32_t)__popc(lm));
+        at = __shfl_sync(FULL, at, 0) + (uint32_t)__popc(lm & ((1u << lane) - 1u));
+        if (list && at < cap) heavy[at] = make_uint2(ca, cb);
+        unsigned om = __ballot_sync(FULL, list && at >= cap);  // list full: linked here
+        while (om) {
+          const int src = __ffs(om) - 1;
+          om &= om - 1;
+          const uint32_t xa = __shfl_sync(FULL, ca, src), xb = __shfl_sync(FULL, cb, src);
+          const u64 ka = lckey[xa], kb = lckey[xb];
+          const int la[3] = {(int)compact3(ka), (int)compact3(ka >> 1), (int)compact3(ka >> 2)};
+          const int lb[3] = {(int)compact3(kb), (int)compact3(kb >> 1), (int)compact3(kb >> 2)};
+          link_cells_warp(f, parent, f.lcfirst[xa], f.lcfirst[xa + 1], la, f.lcfirst[xb],
+                          f.lcfirst[xb + 1], lb, false, (ka & kb & kOneSet) != 0);
+          __syncwarp();
         }
       }
     }
-    while (__any_sync(FULL, cur < (uint32_t)n)) {
-      if (lane == 0) s_cnt[w] = 0;
-      __syncwarp();
-      while (cur < (uint32_t)n) {
-        const u64 bk = keyS[cur];
-        if ((bk >> 6) != nkey) {
-          cur = (uint32_t)n;
-          break;
-        }
-        const int slot = atomicAdd(&s_cnt[w], 1);
-        if (slot >= kLCap) break;  // full: this sub-cell waits for the next round
-        const uint32_t j1 = sc_start[sid[cur] + 1];
-        s_b0[w][slot] = cur;
-        s_b1[w][slot] = j1;
-        s_bc[w][slot] = pack_sub(VR_SUB_OF(bk, nx, ny, nz));
-        cur = j1;
-      }
-      __syncwarp();
-      const int nb = min(s_cnt[w], kLCap);
-      for (int t = lane; t < m * nb; t += 32) {
-        const int i = t / nb, j = t - i * nb;
-        link_pair(posS, parent, s_a0[w][i], s_a0[w][i + 1], s_ac[w][i], s_b0[w][j], s_b1[w][j],
-                  s_bc[w][j], S, T);
-      }
-      __syncwarp();
+    __syncwarp();  // s_task is rewritten for the next 32 cells
+  }
+}
+
+// The listed pairs of link cells, one warp each.
+__global__ void __launch_bounds__(32 * kLW) k_fof_heavy(FofCells f, const u64 *__restrict__ lckey,
+                                                        int *parent, const uint2 *__restrict__ heavy,
+                                                        uint32_t cap, const uint32_t *__restrict__ nheavy) {
+  const uint32_t n = min(*nheavy, cap);
+  for (u64 k = (u64)blockIdx.x * kLW + (threadIdx.x >> 5); k < n; k += (u64)gridDim.x * kLW) {
+    const uint2 c = heavy[k];
+    const u64 ka = lckey[c.x], kb = lckey[c.y];
+    const bool once = (ka & kb & kOneSet) != 0;
+    const uint32_t sa0 = f.lcfirst[c.x], sb0 = f.lcfirst[c.y];
+    if (once) {
+      int same = 0;
+      if ((threadIdx.x & 31) == 0) same = uf_find(parent, (int)sa0) == uf_find(parent, (int)sb0);
+      if (__shfl_sync(0xffffffffu, same, 0)) continue;
     }
-    __syncwarp();  // s_a0 / s_ac are rewritten for the next link cell
-    }
+    const int la[3] = {(int)compact3(ka), (int)compact3(ka >> 1), (int)compact3(ka >> 2)};
+    const int lb[3] = {(int)compact3(kb), (int)compact3(kb >> 1), (int)compact3(kb >> 2)};
+    link_cells_warp(f, parent, sa0, f.lcfirst[c.x + 1], la, sb0, f.lcfirst[c.y + 1], lb, false, once);
+    __syncwarp();
   }
 }
 
 // Root of every particle and the minimum original index per root. Neighbours in sort
 // order mostly share a root, so the lanes of a warp with the same root combine their
 // minimum first and one of them updates the root (one atomic per root and warp).
-__global__ void k_fof_roots(int *parent, const int4 *__restrict__ posS, int64_t n,
-                            int *__restrict__ minidx) {
+__global__ void k_fof_roots(int *parent, const uint32_t *__restrict__ sid,
+                            const int4 *__restrict__ posS, int64_t n, uint32_t *__restrict__ minidx) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const bool valid = p < n;
-  int r = -1 - lane, w = 0x7fffffff;
+  int r = -1 - lane;
+  uint32_t w = 0xffffffffu;
   if (valid) {
-    r = uf_find(parent, (int)p);
-    parent[p] = r;
-    w = posS[p].w;
+    const int s = (int)sid[p];
+    r = uf_find(parent, s);
+    parent[s] = r;
+    w = (uint32_t)posS[p].w;
   }
   const unsigned peers = __match_any_sync(0xffffffffu, r);
-  const int m = __reduce_min_sync(peers, w);
+  const uint32_t m = __reduce_min_sync(peers, w);
   if (valid && lane == __ffs(peers) - 1) atomicMin(&minidx[r], m);
 }
 
-// A fresh find: parent[p] written by k_fof_roots may since have been overwritten by a
+// A fresh find: parent[s] written by k_fof_roots may since have been overwritten by a
 // concurrent path-halving store with an older ancestor, so it is not read directly.
-__global__ void k_fof_label(int *parent, const int4 *__restrict__ posS,
-                            const int *__restrict__ minidx, int64_t n, int32_t *__restrict__ label) {
+__global__ void k_fof_label(int *parent, const uint32_t *__restrict__ sid,
+                            const int4 *__restrict__ posS, const uint32_t *__restrict__ minidx,
+                            int64_t n, int32_t *__restrict__ label) {
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  label[posS[p].w] = minidx[uf_find(parent, (int)p)];
+  label[posS[p].w] = (int32_t)minidx[uf_find(parent, (int)sid[p])];
 }
 
 }  // namespace
@@ -596,38 +670,42 @@ extern "C" vr_status vr_fof3d(vr_ctx *ctx, const int32_t *pos, int64_t n, int64_
                                      &which));
   u64 *keyS = which ? B.k1 : B.k0;
   uint32_t *orig = which ? B.v1 : B.v0;
-  VR_CUDA(ctx, cudaMemsetAsync(B.cstart, 0xff, g.ncoarse * sizeof(uint32_t), s));
+  VR_CUDA(ctx, cudaMemsetAsync(B.ctab, 0xff, g.ncoarse * sizeof(uint2), s));
   VR_CUDA(ctx, cudaMemsetAsync(B.occ, 0, occ_words(g.om) * sizeof(unsigned long long), s));
   const int qshift = 3 * g.q;      // link-cell key -> coarse-cell key
   const int cshift = 6 + qshift;   // sort key -> coarse-cell key
-  k_fof_prepare<<<grid_for(n + 1, T), T, 0, s>>>(pos, keyS, orig, n, cshift, B.posS, B.minidx,
-                                                 B.head, B.cstart, B.cend, B.occ, g.om);
+  u64 *spare = which ? B.k0 : B.k1;
+  k_fof_prepare<<<grid_for(n + 1, T), T, 0, s>>>(pos, keyS, orig, n, B.posS, spare);
   VR_LAUNCHED(ctx, "k_fof_prepare");
-  VR_CUDA(ctx, exclusive_scan<uint32_t>(B.head, B.head, n + 1, B.scratch, s));
+  VR_CUDA(ctx, exclusive_scan<u64>(spare, spare, n + 1, B.scratch, s));
   uint32_t *sid = which ? B.v0 : B.v1;  // the sort's spare value buffer
-  k_fof_subcells<<<grid_for(n, T), T, 0, s>>>(keyS, B.head, n, sid, B.sc_start);
-  VR_LAUNCHED(ctx, "k_fof_subcells");
-  k_fof_hook<<<grid_for(n, T), T, 0, s>>>(sid, B.sc_start, n, B.parent);
-  VR_LAUNCHED(ctx, "k_fof_hook");
-  // link cells as runs of sub-cells, in the sort's spare key buffer (2 n + 2 words):
-  // lcf [0, n] the scanned first-sub-cell flags, lcfirst [n + 1, 2 n + 2) the first
-  // sub-cell of each link cell; the number of sub-cells, head[n], stays on the device
-  uint32_t *lcf = reinterpret_cast<uint32_t *>(which ? B.k0 : B.k1);
-  uint32_t *lcfirst = lcf + (n + 1);
-  k_fof_lcflags<<<grid_for(n + 1, T), T, 0, s>>>(keyS, B.sc_start, B.head + n, n, lcf);
-  VR_LAUNCHED(ctx, "k_fof_lcflags");
-  VR_CUDA(ctx, exclusive_scan<uint32_t>(lcf, lcf, n + 1, B.scratch, s));
-  k_fof_lcfirst<<<grid_for(n + 1, T), T, 0, s>>>(keyS, B.sc_start, B.head + n, n, lcf, lcfirst);
-  VR_LAUNCHED(ctx, "k_fof_lcfirst");
+  uint32_t *lcfirst = orig;             // posS holds the particle indices now
+  k_fof_cells<<<grid_for(n, T), T, 0, s>>>(keyS, spare, n, cshift, sid, B.sc_start, lcfirst, B.lckey,
+                                           B.ctab, B.occ, g.om, B.parent);
+  VR_LAUNCHED(ctx, "k_fof_cells");
   int sms = ctx->sm_count;
   if (sms <= 0) VR_CUDA(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-  VR_TIMED(ctx, "fof_link", s, k_fof_link_w<<<5 * sms, 32 * kLW, 0, s>>>(B.posS, keyS, sid, B.sc_start, lcf, lcfirst, B.cstart,
-                                          B.cend, B.occ, g.om, B.parent, n, g.S, g.GL, qshift,
-                                          (long long)link_d2));
-  VR_LAUNCHED(ctx, "k_fof_link_w");
-  k_fof_roots<<<grid_for(n, T), T, 0, s>>>(B.parent, B.posS, n, B.minidx);
+  // the scanned flags stay until the link kernels have read their last entry; the list of
+  // heavy pairs takes the entries before it
+  uint32_t *nheavy = reinterpret_cast<uint32_t *>(B.scratch);
+  uint2 *heavy = reinterpret_cast<uint2 *>(spare);
+  VR_CUDA(ctx, cudaMemsetAsync(nheavy, 0, sizeof(uint32_t), s));
+  FofCells f{B.posS, keyS, B.sc_start, lcfirst, B.ctab, B.occ, g.om, g.S, g.GL, qshift, (long long)link_d2};
+  const unsigned lgrid = (unsigned)grid_for(n, 32 * kLW, 16LL * sms);
+  timer_begin(ctx, "fof_link", s);
+  k_fof_own<<<lgrid, 32 * kLW, 0, s>>>(f, spare + n, B.lckey, B.parent);
+  VR_LAUNCHED(ctx, "k_fof_own");
+  k_fof_neigh<<<lgrid, 32 * kLW, 0, s>>>(f, spare + n, B.lckey, B.parent, heavy, (uint32_t)n, nheavy);
+  VR_LAUNCHED(ctx, "k_fof_neigh");
+  k_fof_heavy<<<(unsigned)grid_for(n, 32 * kLW, 8LL * sms), 32 * kLW, 0, s>>>(f, B.lckey, B.parent, heavy,
+                                                                            (uint32_t)n, nheavy);
+  VR_LAUNCHED(ctx, "k_fof_heavy");
+  timer_end(ctx, "fof_link", s);
+  uint32_t *minidx = reinterpret_cast<uint32_t *>(spare);  // the list is done
+  VR_CUDA(ctx, cudaMemsetAsync(minidx, 0xff, n * sizeof(uint32_t), s));
+  k_fof_roots<<<grid_for(n, T), T, 0, s>>>(B.parent, sid, B.posS, n, minidx);
   VR_LAUNCHED(ctx, "k_fof_roots");
-  k_fof_label<<<grid_for(n, T), T, 0, s>>>(B.parent, B.posS, B.minidx, n, label);
+  k_fof_label<<<grid_for(n, T), T, 0, s>>>(B.parent, sid, B.posS, minidx, n, label);
   VR_LAUNCHED(ctx, "k_fof_label");
   return log_call(ctx, "vr_fof3d", n, VR_OK);
 }
