@@ -271,14 +271,16 @@ __device__ __forceinline__ uint32_t compact3(u64 x) {  // every third bit of x, 
 // Pairs of sub-cells with at most this many member pairs are tested particle by particle,
 // without the box tests; those of more than kSerialPairs by a whole warp.
 constexpr uint32_t kDirectPairs = 4, kSerialPairs = 64;
-// Link-cell pairs of at most this many member pairs are tested by one lane of k_fof_neigh.
-constexpr uint32_t kLanePairs = 32;
+// Link-cell pairs of at most this many member pairs are tested where they are found, their
+// member pairs spread over the warp; larger ones are listed for a warp of their own.
+constexpr uint32_t kLanePairs = 64;
 constexpr u64 kOneSet = 1ull << 63;  // lckey: the link cell's sub-cells are all in one set
 
 struct FofCells {
   const int4 *posS;
   const u64 *keyS;
   const uint32_t *sc_start, *lcfirst;
+  const uint32_t *sid;
   const uint2 *ctab;
   const unsigned long long *occ;
   int om, S, GL, qshift;
@@ -421,49 +423,104 @@ __device__ void link_cells_warp(const FofCells &f, int *parent, uint32_t sa0, ui
   }
 }
 
-// Pairs of sub-cells of one link cell; lane l of a warp takes link cell c0 + l, the cells
-// of more than kLanePairs member pairs are taken by the whole warp.
+// Tests the member pairs of up to 32 pairs of particle runs, one pair of runs per lane (w =
+// its member pairs, 0: none): the pairs of all lanes follow one another, and each step takes
+// the next 32. Lanes that walked their own few pairs left two thirds of the warp idle
+// (k_fof_neigh at 512^3: 23.0 -> 17.5 ms). A run paired with itself takes i < j only.
+__device__ __forceinline__ void link_runs(const FofCells &f, int *parent, uint32_t a0, uint32_t b0,
+                                          uint32_t nb, uint32_t w) {
+  const int lane = threadIdx.x & 31;
+  const unsigned FULL = 0xffffffffu;
+  uint32_t incl = w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const uint32_t total = __shfl_sync(FULL, incl, 31);
+  for (uint32_t base = 0; base < total; base += 32) {
+    const uint32_t t = base + lane;
+    int o = 0;  // the lane that holds pair t: the first whose inclusive count exceeds it
+#pragma unroll
+    for (int s = 16; s; s >>= 1)
+      if (__shfl_sync(FULL, incl, o + s - 1) <= t) o += s;
+    const uint32_t at = t - __shfl_sync(FULL, incl - w, o), m = __shfl_sync(FULL, nb, o);
+    const uint32_t xa = __shfl_sync(FULL, a0, o), xb = __shfl_sync(FULL, b0, o);
+    if (t < total) {
+      const uint32_t i = at / m, j = at - i * m;
+      const uint32_t a = xa + i, b = xb + j;
+      if ((xa != xb || i < j) && d2_periodic(f.posS[a], f.posS[b]) < f.T) {
+        const int sa = (int)f.sid[a], sb = (int)f.sid[b];
+        if (sa != sb) uf_unite(parent, sa, sb);
+      }
+    }
+  }
+}
+
+// Pairs of sub-cells of one link cell; a warp takes `per` link cells at a time, the cells of
+// more than kLanePairs member pairs go to the list (as pairs with themselves): a run of
+// dense link cells is a run in sort order too, and left with the warp that holds it it was
+// the kernel's last 1 ms at 256^3.
 constexpr int kLW = 4;  // warps per block of the link kernels
 __global__ void __launch_bounds__(32 * kLW) k_fof_own(FofCells f, const u64 *__restrict__ excl_n,
-                                                      u64 *__restrict__ lckey, int *parent) {
+                                                      u64 *__restrict__ lckey, int *parent,
+                                                      uint2 *__restrict__ heavy,
+                                                      uint32_t *__restrict__ nheavy, int per) {
   const int lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
   const int64_t nlc = (uint32_t)*excl_n;
-  for (int64_t c0 = ((int64_t)blockIdx.x * kLW + (threadIdx.x >> 5)) * 32; c0 < nlc;
-       c0 += (int64_t)gridDim.x * kLW * 32) {
-    uint32_t s0 = 0, s1 = 0;
-    bool one = false, many = false;
-    if (c0 + lane < nlc) {
-      s0 = f.lcfirst[c0 + lane];
-      s1 = f.lcfirst[c0 + lane + 1];
-      one = s1 - s0 == 1;
-      if (!one) {
-        const u64 np = f.sc_start[s1] - f.sc_start[s0];
-        many = np * np > 2 * kLanePairs;
-        if (!many) {
-          for (uint32_t i = s0; i < s1; ++i)
-            for (uint32_t j = i + 1; j < s1; ++j)
-              if (any_pair(f, f.sc_start[i], f.sc_start[i + 1], f.sc_start[j], f.sc_start[j + 1]))
-                uf_unite(parent, (int)i, (int)j);
-        }
+  for (int64_t c0 = ((int64_t)blockIdx.x * kLW + (threadIdx.x >> 5)) * per; c0 < nlc;
+       c0 += (int64_t)gridDim.x * kLW * per) {
+    const int64_t c = c0 + lane;
+    uint32_t s0 = 0, s1 = 0, p0 = 0, np = 0, w = 0;
+    if (lane < per && c < nlc) {
+      s0 = f.lcfirst[c];
+      s1 = f.lcfirst[c + 1];
+      if (s1 - s0 > 1) {
+        p0 = f.sc_start[s0];
+        np = f.sc_start[s1] - p0;
+        w = (u64)np * np > 2 * kLanePairs ? 0 : np * np;
       }
     }
-    unsigned mm = __ballot_sync(FULL, many);
-    while (mm) {
-      const int src = __ffs(mm) - 1;
-      mm &= mm - 1;
-      const uint32_t a = __shfl_sync(FULL, s0, src), b = __shfl_sync(FULL, s1, src);
-      const u64 k = lckey[c0 + src];
-      const int l[3] = {(int)compact3(k), (int)compact3(k >> 1), (int)compact3(k >> 2)};
-      link_cells_warp(f, parent, a, b, l, a, b, l, true, false);
+    const unsigned lm = __ballot_sync(FULL, np > 0 && w == 0);
+    if (lm) {
+      uint32_t at = 0;
+      if (lane == 0) at = atomicAdd(nheavy, (uint32_t)__popc(lm));
+      at = __shfl_sync(FULL, at, 0) + (uint32_t)__popc(lm & ((1u << lane) - 1u));
+      if (np > 0 && w == 0) heavy[at] = make_uint2((uint32_t)c, (uint32_t)c);  // at most one per cell
+    }
+    if (__any_sync(FULL, w > 0)) {
+      link_runs(f, parent, p0, p0, np > 0 ? np : 1, w);
       __syncwarp();
     }
-    if (s1 - s0 > 1) {  // one set: every sub-cell has the first one's root
+    bool one = s1 - s0 == 1;
+    if (w > 0) {  // one set: every sub-cell has the first one's root
       const int r = uf_find(parent, (int)s0);
       one = true;
       for (uint32_t i = s0 + 1; i < s1 && one; ++i) one = uf_find(parent, (int)i) == r;
     }
-    if (one) lckey[c0 + lane] |= kOneSet;
+    if (one) lckey[c] |= kOneSet;
+  }
+}
+
+// The listed link cells, one warp each.
+__global__ void __launch_bounds__(32 * kLW) k_fof_own_heavy(FofCells f, u64 *__restrict__ lckey,
+                                                            int *parent, const uint2 *__restrict__ heavy,
+                                                            const uint32_t *__restrict__ nheavy) {
+  const int lane = threadIdx.x & 31;
+  const unsigned FULL = 0xffffffffu;
+  const uint32_t n = *nheavy;
+  for (u64 k = (u64)blockIdx.x * kLW + (threadIdx.x >> 5); k < n; k += (u64)gridDim.x * kLW) {
+    const uint32_t c = heavy[k].x;
+    const uint32_t s0 = f.lcfirst[c], s1 = f.lcfirst[c + 1];
+    const u64 key = lckey[c];
+    const int l[3] = {(int)compact3(key), (int)compact3(key >> 1), (int)compact3(key >> 2)};
+    link_cells_warp(f, parent, s0, s1, l, s0, s1, l, true, false);
+    __syncwarp();
+    bool one = true;
+    const int r = uf_find(parent, (int)s0);
+    for (uint32_t i = s0 + lane; i < s1; i += 32) one = one && uf_find(parent, (int)i) == r;
+    if (__all_sync(FULL, one) && lane == 0) lckey[c] = key | kOneSet;
   }
 }
 
@@ -487,21 +544,26 @@ __device__ __forceinline__ void fwd_cell(const int *l, int q, int GL, int *o) {
   }
 }
 
-// Pairs of adjacent link cells, as described at the top. Each warp takes 32 consecutive
-// link cells at a time.
-__global__ void __launch_bounds__(32 * kLW) k_fof_neigh(FofCells f, const u64 *__restrict__ excl_n,
+// Pairs of adjacent link cells, as described at the top. Each warp takes `per` consecutive
+// link cells at a time: 32, fewer for a small box, whose few link cells would leave most
+// warp slots empty (32^3: 197 -> 67 us).
+__global__ void __launch_bounds__(32 * kLW, 12) k_fof_neigh(FofCells f, const u64 *__restrict__ excl_n,
                                                         const u64 *__restrict__ lckey, int *parent,
                                                         uint2 *__restrict__ heavy, uint32_t cap,
-                                                        uint32_t *__restrict__ nheavy) {
+                                                        uint32_t *__restrict__ nheavy, int per) {
   __shared__ uint16_t s_task[kLW][32 * 13];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned FULL = 0xffffffffu;
   const int64_t nlc = (uint32_t)*excl_n;
-  for (int64_t c0 = ((int64_t)blockIdx.x * kLW + w) * 32; c0 < nlc; c0 += (int64_t)gridDim.x * kLW * 32) {
+  for (int64_t c0 = ((int64_t)blockIdx.x * kLW + w) * per; c0 < nlc; c0 += (int64_t)gridDim.x * kLW * per) {
     uint32_t bits = 0;
-    if (c0 + lane < nlc) {
-      const u64 k = lckey[c0 + lane];
-      const int l[3] = {(int)compact3(k), (int)compact3(k >> 1), (int)compact3(k >> 2)};
+    int l[3] = {0, 0, 0};
+    u64 k = 0;
+    if (lane < per && c0 + lane < nlc) {
+      k = lckey[c0 + lane];
+      l[0] = (int)compact3(k);
+      l[1] = (int)compact3(k >> 1);
+      l[2] = (int)compact3(k >> 2);
 #pragma unroll
       for (int q = 0; q < 13; ++q) {
         int o[3];
@@ -525,15 +587,16 @@ __global__ void __launch_bounds__(32 * kLW) k_fof_neigh(FofCells f, const u64 *_
     __syncwarp();
     for (int t0 = 0; t0 < ntask; t0 += 32) {
       const int t = t0 + lane;
-      uint32_t ca = 0, cb = kEmpty;
+      uint32_t ca = 0, cb = kEmpty, p0 = 0, q0 = 0, nq = 1, wk = 0;
       bool list = false;
+      const int task = t < ntask ? s_task[w][t] : 0;
+      const u64 ka = __shfl_sync(FULL, k, task >> 4);
+      const int la[3] = {__shfl_sync(FULL, l[0], task >> 4), __shfl_sync(FULL, l[1], task >> 4),
+                         __shfl_sync(FULL, l[2], task >> 4)};
       if (t < ntask) {
-        const int task = s_task[w][t];
         ca = (uint32_t)c0 + (uint32_t)(task >> 4);
-        const u64 ka = lckey[ca];
-        const int l[3] = {(int)compact3(ka), (int)compact3(ka >> 1), (int)compact3(ka >> 2)};
         int o[3];
-        fwd_cell(l, task & 15, f.GL, o);
+        fwd_cell(la, task & 15, f.GL, o);
         cb = find_cell(f, lckey, morton3((uint32_t)o[0], (uint32_t)o[1], (uint32_t)o[2]));
         if (cb != kEmpty) {
           const bool once = (ka & __ldg(&lckey[cb]) & kOneSet) != 0;
@@ -545,19 +608,17 @@ __global__ void __launch_bounds__(32 * kLW) k_fof_neigh(FofCells f, const u64 *_
             if (d2_periodic(f.posS[a0], f.posS[b0]) < f.T) uf_unite(parent, (int)sa0, (int)sb0);
           } else if (!(once && uf_find(parent, (int)sa0) == uf_find(parent, (int)sb0))) {
             if ((u64)(a1 - a0) * (b1 - b0) <= kLanePairs) {
-              bool done = false;
-              for (uint32_t i = sa0; i < sa1 && !done; ++i)
-                for (uint32_t j = sb0; j < sb1 && !done; ++j)
-                  if (any_pair(f, f.sc_start[i], f.sc_start[i + 1], f.sc_start[j], f.sc_start[j + 1])) {
-                    uf_unite(parent, (int)i, (int)j);
-                    done = once;
-                  }
+              p0 = a0;
+              q0 = b0;
+              nq = b1 - b0;
+              wk = (a1 - a0) * nq;
             } else {
               list = true;
             }
           }
         }
       }
+      if (__any_sync(FULL, wk > 0)) link_runs(f, parent, p0, q0, nq, wk);
       const unsigned lm = __ballot_sync(FULL, list);
       if (lm) {
         uint32_t at = 0;
@@ -569,11 +630,11 @@ __global__ void __launch_bounds__(32 * kLW) k_fof_neigh(FofCells f, const u64 *_
           const int src = __ffs(om) - 1;
           om &= om - 1;
           const uint32_t xa = __shfl_sync(FULL, ca, src), xb = __shfl_sync(FULL, cb, src);
-          const u64 ka = lckey[xa], kb = lckey[xb];
-          const int la[3] = {(int)compact3(ka), (int)compact3(ka >> 1), (int)compact3(ka >> 2)};
-          const int lb[3] = {(int)compact3(kb), (int)compact3(kb >> 1), (int)compact3(kb >> 2)};
-          link_cells_warp(f, parent, f.lcfirst[xa], f.lcfirst[xa + 1], la, f.lcfirst[xb],
-                          f.lcfirst[xb + 1], lb, false, (ka & kb & kOneSet) != 0);
+          const u64 k0 = lckey[xa], k1 = lckey[xb];
+          const int x0[3] = {(int)compact3(k0), (int)compact3(k0 >> 1), (int)compact3(k0 >> 2)};
+          const int x1[3] = {(int)compact3(k1), (int)compact3(k1 >> 1), (int)compact3(k1 >> 2)};
+          link_cells_warp(f, parent, f.lcfirst[xa], f.lcfirst[xa + 1], x0, f.lcfirst[xb],
+                          f.lcfirst[xb + 1], x1, false, (k0 & k1 & kOneSet) != 0);
           __syncwarp();
         }
       }
@@ -689,16 +750,25 @@ extern "C" vr_status vr_fof3d(vr_ctx *ctx, const int32_t *pos, int64_t n, int64_
   // heavy pairs takes the entries before it
   uint32_t *nheavy = reinterpret_cast<uint32_t *>(B.scratch);
   uint2 *heavy = reinterpret_cast<uint2 *>(spare);
-  VR_CUDA(ctx, cudaMemsetAsync(nheavy, 0, sizeof(uint32_t), s));
-  FofCells f{B.posS, keyS, B.sc_start, lcfirst, B.ctab, B.occ, g.om, g.S, g.GL, qshift, (long long)link_d2};
-  const unsigned lgrid = (unsigned)grid_for(n, 32 * kLW, 16LL * sms);
+  VR_CUDA(ctx, cudaMemsetAsync(nheavy, 0, 2 * sizeof(uint32_t), s));
+  FofCells f{B.posS, keyS, B.sc_start, lcfirst, sid, B.ctab, B.occ, g.om, g.S, g.GL, qshift, (long long)link_d2};
+  // link cells a warp takes at a time (n bounds their number): 32, or 64 warps per SM. Each
+  // warp takes two such runs; more blocks than fit at once let the dense regions, which lie
+  // together in sort order, spread over the SMs (k_fof_neigh at 512^3 with the resident
+  // blocks only 17.5 ms, now 13.1 ms)
+  int per = 4;
+  while (per < 32 && n > 64LL * sms * per) per *= 2;
+  const unsigned hgrid = (unsigned)grid_for(n, 32 * kLW, 64LL * sms);
   timer_begin(ctx, "fof_link", s);
-  k_fof_own<<<lgrid, 32 * kLW, 0, s>>>(f, spare + n, B.lckey, B.parent);
+  k_fof_own<<<(unsigned)grid_for(n, 2 * per * kLW), 32 * kLW, 0, s>>>(f, spare + n, B.lckey, B.parent,
+                                                                           heavy, nheavy, per);
   VR_LAUNCHED(ctx, "k_fof_own");
-  k_fof_neigh<<<lgrid, 32 * kLW, 0, s>>>(f, spare + n, B.lckey, B.parent, heavy, (uint32_t)n, nheavy);
+  k_fof_own_heavy<<<hgrid, 32 * kLW, 0, s>>>(f, B.lckey, B.parent, heavy, nheavy);
+  VR_LAUNCHED(ctx, "k_fof_own_heavy");
+  k_fof_neigh<<<(unsigned)grid_for(n, 2 * per * kLW), 32 * kLW, 0, s>>>(
+      f, spare + n, B.lckey, B.parent, heavy, (uint32_t)n, nheavy + 1, per);
   VR_LAUNCHED(ctx, "k_fof_neigh");
-  k_fof_heavy<<<(unsigned)grid_for(n, 32 * kLW, 8LL * sms), 32 * kLW, 0, s>>>(f, B.lckey, B.parent, heavy,
-                                                                            (uint32_t)n, nheavy);
+  k_fof_heavy<<<hgrid, 32 * kLW, 0, s>>>(f, B.lckey, B.parent, heavy, (uint32_t)n, nheavy + 1);
   VR_LAUNCHED(ctx, "k_fof_heavy");
   timer_end(ctx, "fof_link", s);
   uint32_t *minidx = reinterpret_cast<uint32_t *>(spare);  // the list is done
