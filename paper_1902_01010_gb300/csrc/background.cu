@@ -28,7 +28,9 @@ namespace vr {
 
 namespace {
 
-constexpr int kFrameT = 256;       // threads per halo-frame CTA
+constexpr int kFrameT = 256;       // threads per halo-frame CTA, halos below kFrameBig
+constexpr int kFrameTBig = 1024;   // and of kFrameBig members or more
+constexpr uint32_t kFrameBig = 16384;
 constexpr int kSmallT = 256;       // threads per tree-building CTA, halos below kBigHalo
 constexpr int kBigT = 1024;        // threads per tree-building CTA, halos of kBigHalo or more
 constexpr int64_t kBigHalo = 65536;
@@ -73,35 +75,41 @@ __device__ __forceinline__ int coord(const int4 &p, int a) { return a == 0 ? p.x
 
 }  // namespace
 
-// Halo table row for every halo (searched or not): FP64 frame and sigma_host.
-__global__ void __launch_bounds__(kFrameT) k_halo_frame(const uint32_t *__restrict__ hoff,
+// Halo table row for every halo (searched or not): FP64 frame and sigma_host. Two passes over
+// a halo's velocities, bound by their latency: the blocks of large halos have 1,024 threads
+// and every thread four loads in flight (@FRAME@).
+template <int NT>
+__global__ void __launch_bounds__(NT) k_halo_frame(const uint32_t *__restrict__ hoff,
                                                     const uint32_t *__restrict__ hlabel,
                                                     const uint32_t *__restrict__ horder, int64_t first,
                                                     int64_t last, const float4 *__restrict__ v,
                                                     int nsearch_min, double *__restrict__ hs_out) {
-  __shared__ double sd[kFrameT / 32];
+  __shared__ double sd[NT / 32];
   if (first + (int64_t)blockIdx.x >= last) return;
   const int64_t h = horder[first + blockIdx.x];  // largest halos first
   const uint32_t b = hoff[h], e = hoff[h + 1];
+  if ((NT == kFrameTBig) != (e - b >= kFrameBig)) return;  // each size class has its own launch
   const double nh = (double)(e - b);
   double s[3] = {0, 0, 0};
-  for (uint32_t m = b + threadIdx.x; m < e; m += kFrameT) {
+#pragma unroll 4
+  for (uint32_t m = b + threadIdx.x; m < e; m += NT) {
     float4 q = v[m];
     s[0] += (double)q.x;
     s[1] += (double)q.y;
     s[2] += (double)q.z;
   }
   double mean[3];
-  for (int k = 0; k < 3; ++k) mean[k] = block_reduce<kFrameT>(s[k], AddD(), sd) / nh;
+  for (int k = 0; k < 3; ++k) mean[k] = block_reduce<NT>(s[k], AddD(), sd) / nh;
   double c[6] = {0, 0, 0, 0, 0, 0};
-  for (uint32_t m = b + threadIdx.x; m < e; m += kFrameT) {
+#pragma unroll 4
+  for (uint32_t m = b + threadIdx.x; m < e; m += NT) {
     float4 q = v[m];
     double d0 = (double)q.x - mean[0], d1 = (double)q.y - mean[1], d2 = (double)q.z - mean[2];
     c[0] += d0 * d0; c[1] += d1 * d1; c[2] += d2 * d2;
     c[3] += d0 * d1; c[4] += d0 * d2; c[5] += d1 * d2;
   }
   double S[6];
-  for (int k = 0; k < 6; ++k) S[k] = block_reduce<kFrameT>(c[k], AddD(), sd) / nh;
+  for (int k = 0; k < 6; ++k) S[k] = block_reduce<NT>(c[k], AddD(), sd) / nh;
   if (threadIdx.x == 0) {
     double det = S[0] * (S[1] * S[2] - S[5] * S[5]) - S[3] * (S[3] * S[2] - S[5] * S[4]) +
                  S[4] * (S[3] * S[5] - S[1] * S[4]);
@@ -124,9 +132,18 @@ __global__ void __launch_bounds__(kFrameT) k_halo_frame(const uint32_t *__restri
 vr_status run_halo_frame(vr_ctx *ctx, const HaloSeg &g, int nsearch_min, double *halo_stats,
                          cudaStream_t s) {
   if (g.H == 0) return VR_OK;
-  VR_TIMED(ctx, "halo_frame", s, k_halo_frame<<<(unsigned)g.H, kFrameT, 0, s>>>(
-      g.hoff, g.hlabel, g.horder, 0, g.H, g.v, nsearch_min, halo_stats));
+  // the large halos are the first of the size order, at most NHP / kFrameBig of them
+  const int64_t nbig = g.NHP / kFrameBig < g.H ? g.NHP / kFrameBig : g.H;
+  timer_begin(ctx, "halo_frame", s);
+  if (nbig > 0) {
+    k_halo_frame<kFrameTBig><<<(unsigned)nbig, kFrameTBig, 0, s>>>(g.hoff, g.hlabel, g.horder, 0, nbig, g.v,
+                                                                  nsearch_min, halo_stats);
+    VR_LAUNCHED(ctx, "k_halo_frame<big>");
+  }
+  k_halo_frame<kFrameT><<<(unsigned)g.H, kFrameT, 0, s>>>(g.hoff, g.hlabel, g.horder, 0, g.H, g.v, nsearch_min,
+                                                         halo_stats);
   VR_LAUNCHED(ctx, "k_halo_frame");
+  timer_end(ctx, "halo_frame", s);
   return VR_OK;
 }
 
@@ -863,7 +880,7 @@ vr_status run_background(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Aren
   int64_t hmax = g.n / (p->nmin > 0 ? p->nmin : 1) + 2;
   Background &bg = *out;
   bg.nodeoff = ar.take<uint32_t>(hmax + 1);
-  uint32_t *perm = ar.take<uint32_t>(g.n);
+  uint32_t *perm = bg.scratch = ar.take<uint32_t>(g.n);
   uint32_t *tmp = ar.take<uint32_t>(g.n);
   bg.leaf_of = ar.take<uint32_t>(g.n);
   int64_t cap = max_nodes(g.n, p);
@@ -874,8 +891,13 @@ vr_status run_background(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Aren
   if (H == 0) return VR_OK;
   if (hoff_host) {
     for (int64_t i = 0; i < H; ++i) {
-      k_halo_frame<<<1, kFrameT, 0, s>>>(g.hoff, g.hlabel, g.horder, i, i + 1, g.v, p->nsearch_min,
-                                         halo_stats);
+      if (i < g.NHP / kFrameBig) {  // may be a large one (its own kernel skips the others)
+        k_halo_frame<kFrameTBig><<<1, kFrameTBig, 0, s>>>(g.hoff, g.hlabel, g.horder, i, i + 1, g.v,
+                                                          p->nsearch_min, halo_stats);
+        VR_LAUNCHED(ctx, "k_halo_frame<big>");
+      }
+      k_halo_frame<kFrameT><<<1, kFrameT, 0, s>>>(g.hoff, g.hlabel, g.horder, i, i + 1, g.v, p->nsearch_min,
+                                                  halo_stats);
       VR_LAUNCHED(ctx, "k_halo_frame");
     }
   } else {

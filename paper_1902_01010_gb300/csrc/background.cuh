@@ -21,6 +21,7 @@ struct Background {
   uint32_t *nodeoff;  // [H+1] first node slot of each halo (0-width for unsearched halos)
   uint32_t *leaf_of;  // [NHP] absolute node index of each member's leaf
   CellNode *nodes;
+  uint32_t *scratch;  // [n] the build's permutation; free for later stages
   double *mom;        // [nodes][13]: mass, xbar[3], vbar[3], sigma (xx yy zz xy xz yz)
 };
 

@@ -160,23 +160,32 @@ __device__ __forceinline__ bool fits32(int4 alo, int4 ahi, int4 blo, int4 bhi) {
 __device__ __forceinline__ uint32_t clamp32(u64 x) { return x > 0xffffffffull ? 0xffffffffu : (uint32_t)x; }
 
 // ---------------------------------------------------------------- small halos
+// Halos of at most N_se members: every member is a neighbour. A warp takes 32 consecutive
+// slots of [m0, m1), a lane per slot, and the halos they belong to one after the other: the
+// halo's members are staged 32 at a time and offered to its lanes. The offers are a serial
+// chain, so the work is cut by slots and not by halos: a warp per halo made the 8 x 256
+// offers of a 256-member halo one after the other (@SMALL@).
 template <int NVM>
 __global__ void __launch_bounds__(32 * kWarps) k_velden_small(
-    const uint32_t *__restrict__ hoff, int64_t h0, int64_t h1, const float4 *__restrict__ v,
-    int nse, int nv, float *__restrict__ f_l) {
+    const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ hid, int64_t m0, int64_t m1,
+    const float4 *__restrict__ v, int nse, int nv, float *__restrict__ f_l) {
   __shared__ SmallSmem<NVM> sm[kWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t h = h0 + (int64_t)blockIdx.x * kWarps + w;  // halos [h0, h1)
-  if (h >= h1) return;
-  const uint32_t hs = hoff[h], he = hoff[h + 1];
-  const int nh = (int)(he - hs);
-  if (nh > nse) return;
-  const int nv_eff = nv < nh ? nv : nh;
+  const int64_t s0 = m0 + ((int64_t)blockIdx.x * kWarps + w) * 32;
+  if (s0 >= m1) return;
+  const int64_t k = s0 + lane;
+  const uint32_t h = hid[k < m1 ? k : m1 - 1];
+  unsigned todo = __ballot_sync(0xffffffffu, k < m1);
   float(*top)[32] = sm[w].top;
-  for (uint32_t qb = hs; qb < he; qb += 32) {
-    const uint32_t k = qb + lane;
-    const bool valid = k < he;
-    const float4 vq = v[valid ? k : hs];
+  while (todo) {
+    const uint32_t hh = __shfl_sync(0xffffffffu, h, __ffs(todo) - 1);
+    const bool mine = k < m1 && h == hh;
+    todo &= ~__ballot_sync(0xffffffffu, mine);
+    const uint32_t hs = hoff[hh], he = hoff[hh + 1];
+    const int nh = (int)(he - hs);
+    if (nh > nse) continue;
+    const int nv_eff = nv < nh ? nv : nh;
+    const float4 vq = v[mine ? k : hs];
     TopV t = {0, 0, 0.0f};
     for (uint32_t jb = hs; jb < he; jb += 32) {
       const uint32_t j = jb + lane;
@@ -184,10 +193,10 @@ __global__ void __launch_bounds__(32 * kWarps) k_velden_small(
       if (j < he) sm[w].sv[lane] = v[j];
       __syncwarp();
       const int cnt = (int)min(32u, he - jb);
-      if (valid)
+      if (mine)
         for (int tt = 0; tt < cnt; ++tt) top_insert(top, lane, t, nv_eff, dv2f(sm[w].sv[tt], vq));
     }
-    if (valid) f_l[__float_as_int(vq.w)] = top_density(top, lane, t, nh);
+    if (mine) f_l[__float_as_int(vq.w)] = top_density(top, lane, t, nh);
   }
 }
 
@@ -718,19 +727,20 @@ vr_status run_velden(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &a
   const int T = 256;
   // small halos: all members are neighbours
   auto small = [&](int64_t a, int64_t z) {
+    const int grid = grid_for(z - a, 32 * kWarps);
     if (p->nv <= 32)
-      k_velden_small<32><<<grid_for(z - a, kWarps), 32 * kWarps, 0, s>>>(g.hoff, a, z, g.v, p->nse, p->nv, f_l);
+      k_velden_small<32><<<grid, 32 * kWarps, 0, s>>>(g.hoff, g.hid, a, z, g.v, p->nse, p->nv, f_l);
     else
-      k_velden_small<kNVMax><<<grid_for(z - a, kWarps), 32 * kWarps, 0, s>>>(g.hoff, a, z, g.v, p->nse, p->nv, f_l);
+      k_velden_small<kNVMax><<<grid, 32 * kWarps, 0, s>>>(g.hoff, g.hid, a, z, g.v, p->nse, p->nv, f_l);
   };
   if (hoff_host) {  // one launch per halo
     for (int64_t h = 0; h < H; ++h) {
       if (hoff_host[h + 1] - hoff_host[h] > (uint32_t)p->nse) continue;
-      small(h, h + 1);
+      small(hoff_host[h], hoff_host[h + 1]);
       VR_LAUNCHED(ctx, "k_velden_small");
     }
   } else {
-    VR_TIMED(ctx, "velden_small", s, small(0, H));
+    VR_TIMED(ctx, "velden_small", s, small(0, g.NHP));
     VR_LAUNCHED(ctx, "k_velden_small");
   }
   k_sb_count<<<grid_for(H + 1, T), T, 0, s>>>(g.hoff, g.horder, H, p->nse, sbr);
