@@ -164,7 +164,8 @@ __device__ __forceinline__ uint32_t clamp32(u64 x) { return x > 0xffffffffull ? 
 // slots of [m0, m1), a lane per slot, and the halos they belong to one after the other: the
 // halo's members are staged 32 at a time and offered to its lanes. The offers are a serial
 // chain, so the work is cut by slots and not by halos: a warp per halo made the 8 x 256
-// offers of a 256-member halo one after the other (@SMALL@).
+// offers of a 256-member halo one after the other (660 us, the
+// same for a 32^3 and a 100^3 box; now 115 us).
 template <int NVM>
 __global__ void __launch_bounds__(32 * kWarps) k_velden_small(
     const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ hid, int64_t m0, int64_t m1,
