@@ -17,8 +17,12 @@
 // Cholesky and D^2 use explicitly rounded FP64 operations in the order of the formulas.
 #include <math.h>
 
+#include <cooperative_groups.h>
+
 #include "stages.h"
 #include "vr_workspace.h"
+
+namespace cg = cooperative_groups;
 
 namespace vr {
 
@@ -90,25 +94,32 @@ __device__ __forceinline__ double dist_scalar(const double *__restrict__ S, cons
   return __dadd_rn(__ddiv_rn(a, sx2), __ddiv_rn(b, sv2));
 }
 
-// Block sum of NV doubles per thread, fixed order; the result is valid in thread 0.
-template <int NV>
-__device__ void block_sum(double *x, double (*red)[kCT / 32]) {
+// Sums of NV doubles over the threads of a block (TEAM 1) or of the cluster's TEAM blocks, fixed
+// order, to every thread. `red` and `tot` are used once per kernel.
+template <int NV, int TEAM>
+__device__ void team_sum(double *x, double (*red)[kCT / 32], double *tot) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < NV; ++k)
+  for (int k = 0; k < NV; ++k) {
     for (int o = 16; o; o >>= 1) x[k] += __shfl_down_sync(0xffffffffu, x[k], o);
+    if (lane == 0) red[k][w] = x[k];
+  }
   __syncthreads();
-  if (lane == 0)
+  if (threadIdx.x < NV) {
+    double s = red[threadIdx.x][0];
+    for (int q = 1; q < kCT / 32; ++q) s += red[threadIdx.x][q];
+    tot[threadIdx.x] = s;
+  }
+  if (TEAM > 1) cg::this_cluster().sync(); else __syncthreads();
 #pragma unroll
-    for (int k = 0; k < NV; ++k) red[k][w] = x[k];
-  __syncthreads();
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double t = red[k][0];
-      for (int q = 1; q < kCT / 32; ++q) t += red[k][q];
-      x[k] = t;
+  for (int k = 0; k < NV; ++k) {
+    double s = tot[k];
+    if (TEAM > 1) {
+      s = cg::this_cluster().map_shared_rank(tot, 0)[k];
+      for (int q = 1; q < TEAM; ++q) s += cg::this_cluster().map_shared_rank(tot, q)[k];
     }
+    x[k] = s;
+  }
 }
 
 __global__ void k_cg_roots(const float4 *__restrict__ v, int64_t nhp, const int32_t *__restrict__ core,
@@ -147,17 +158,15 @@ __global__ void k_cg_slots(const float4 *__restrict__ v, int64_t nhp, const int3
   gc[m] = c >= 0 ? cid_of[c] : -1;
 }
 
-// One CTA per core: mean and tensor of the members whose current core is k (Eqs.
-// coremeanphase, coredispphase), its Cholesky factor, and with `clean` set the cleaning
-// of Eq. coresig. With l >= 0 only cores active at level l are recomputed.
-__global__ void __launch_bounds__(kCT) k_cg_moments(
-    const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ pre, const int4 *__restrict__ u,
-    const float4 *__restrict__ v, const int32_t *__restrict__ gc, const int32_t *__restrict__ searched,
-    CoreTab t, int l, int clean, double beta_c) {
-  __shared__ double red[21][kCT / 32];
-  __shared__ double smean[6];
-  const int k = blockIdx.x;
-  if (l >= 0 && !(t.alive[k] && (t.prim[k] || t.level[k] >= l))) return;
+// Mean and tensor of the members whose current core is k (Eqs. coremeanphase,
+// coredispphase), its Cholesky factor, and with `clean` set the cleaning of Eq. coresig, by
+// block `part` of TEAM.
+template <int TEAM>
+__device__ __forceinline__ void core_moments(
+    int k, int part, const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ pre,
+    const int4 *__restrict__ u, const float4 *__restrict__ v, const int32_t *__restrict__ gc,
+    const int32_t *__restrict__ searched, const CoreTab &t, int clean, double beta_c) {
+  __shared__ double s_r1[14][kCT / 32], s_r2[21][kCT / 32], s_t1[14], s_t2[21];
   const int h = t.halo[k];
   const uint32_t s0 = hoff[h], s1 = hoff[h + 1];
   const bool with_p = clean && !t.prim[k];
@@ -170,7 +179,7 @@ __global__ void __launch_bounds__(kCT) k_cg_moments(
   double acc[13];
 #pragma unroll
   for (int a = 0; a < 13; ++a) acc[a] = 0.0;
-  for (uint32_t m = s0 + threadIdx.x; m < s1; m += kCT) {
+  for (uint32_t m = s0 + part * kCT + threadIdx.x; m < s1; m += kCT * TEAM) {
     const int c = gc[m];
     const bool in = c == k;
     const bool inp = with_p && (c == pk || searched[__float_as_int(v[m].w)] >= lp);
@@ -190,7 +199,7 @@ __global__ void __launch_bounds__(kCT) k_cg_moments(
   // the primary group's count rides in the reduction too
   double pc = 0.0;
   if (with_p)
-    for (uint32_t m = s0 + threadIdx.x; m < s1; m += kCT) {
+    for (uint32_t m = s0 + part * kCT + threadIdx.x; m < s1; m += kCT * TEAM) {
       const int c = gc[m];
       pc += (c == pk || searched[__float_as_int(v[m].w)] >= lp) ? 1.0 : 0.0;
     }
@@ -198,19 +207,15 @@ __global__ void __launch_bounds__(kCT) k_cg_moments(
 #pragma unroll
   for (int a = 0; a < 13; ++a) x14[a] = acc[a];
   x14[13] = pc;
-  block_sum<14>(x14, red);
+  team_sum<14, TEAM>(x14, s_r1, s_t1);
   const double M = x14[12];
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int a = 0; a < 6; ++a) smean[a] = x14[a] / M;
-  __syncthreads();
   double mean[6];
 #pragma unroll
-  for (int a = 0; a < 6; ++a) mean[a] = smean[a];
+  for (int a = 0; a < 6; ++a) mean[a] = x14[a] / M;
   double c2[21];
 #pragma unroll
   for (int a = 0; a < 21; ++a) c2[a] = 0.0;
-  for (uint32_t m = s0 + threadIdx.x; m < s1; m += kCT) {
+  for (uint32_t m = s0 + part * kCT + threadIdx.x; m < s1; m += kCT * TEAM) {
     if (gc[m] != k) continue;
     double X[6];
     load_x(u, v, m, X);
@@ -222,8 +227,8 @@ __global__ void __launch_bounds__(kCT) k_cg_moments(
 #pragma unroll
       for (int j = 0; j <= i; ++j) c2[tri(i, j)] += d[i] * d[j];
   }
-  block_sum<21>(c2, red);
-  if (threadIdx.x != 0) return;
+  team_sum<21, TEAM>(c2, s_r2, s_t2);
+  if (part != 0 || threadIdx.x != 0) return;
   double S[21], L[21];
 #pragma unroll
   for (int a = 0; a < 21; ++a) S[a] = c2[a] / M;
@@ -246,6 +251,27 @@ __global__ void __launch_bounds__(kCT) k_cg_moments(
       for (int a = 0; a < 6; ++a) d[a] = x14[6 + a] / Mp - mean[a];
       t.alive[k] = pd && Mp > 0.0 && dist6(L, d) >= beta_c;
     }
+  }
+}
+
+// A cluster per core. The sums are FP64 (some 45 operations a member, of which an SM does two
+// lanes a cycle) over the whole halo's slots, twice, so the blocks share the halos of kTeamHalo
+// members and more; a smaller one is left to the first block (128^3 box, six
+// launches: 2.91 -> 2.01 ms). With l >= 0 only
+// cores that are active at level l are recomputed, in halos that grow.
+constexpr int kCoreTeam = 8;
+constexpr uint32_t kTeamHalo = 4096;
+__global__ void __launch_bounds__(kCT) __cluster_dims__(kCoreTeam, 1, 1) k_cg_moments(
+    const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ pre, const int4 *__restrict__ u,
+    const float4 *__restrict__ v, const int32_t *__restrict__ gc, const int32_t *__restrict__ searched,
+    CoreTab t, int l, const int *__restrict__ hgrow, int clean, double beta_c) {
+  const int k = (int)(blockIdx.x / kCoreTeam), part = (int)(blockIdx.x % kCoreTeam);
+  if (l >= 0 && !(t.alive[k] && (t.prim[k] || t.level[k] >= l) && hgrow[t.halo[k]])) return;
+  if (hoff[t.halo[k] + 1] - hoff[t.halo[k]] >= kTeamHalo) {
+    core_moments<kCoreTeam>(k, part, hoff, pre, u, v, gc, searched, t, clean, beta_c);
+    cg::this_cluster().sync();  // the others may still read this block's sums
+  } else if (part == 0) {
+    core_moments<1>(k, 0, hoff, pre, u, v, gc, searched, t, clean, beta_c);
   }
 }
 
@@ -369,16 +395,16 @@ vr_status run_core_grow(vr_ctx *ctx, const HaloSeg &g, const vr_core_params *cp,
   k_cg_slots<<<grid_for(NHP, T), T, 0, s>>>(g.v, NHP, core, cid_of, gc);
   VR_LAUNCHED(ctx, "k_cg_slots");
   // the cores as found, and the cleaning
-  VR_TIMED(ctx, "core_grow", s, k_cg_moments<<<(unsigned)K, kCT, 0, s>>>(
-      g.hoff, pre, g.u, g.v, gc, ex.searched, t, -1, 1, gp->beta_c));
+  VR_TIMED(ctx, "core_grow", s, k_cg_moments<<<(unsigned)(kCoreTeam * K), kCT, 0, s>>>(
+      g.hoff, pre, g.u, g.v, gc, ex.searched, t, -1, hgrow, 1, gp->beta_c));
   VR_LAUNCHED(ctx, "k_cg_moments");
   VR_CUDA(ctx, cudaMemsetAsync(hgrow, 0, H * sizeof(int), s));
   k_cg_drop<<<grid_for(NHP, T), T, 0, s>>>(NHP, g.hid, t, gc, hgrow);
   VR_LAUNCHED(ctx, "k_cg_drop");
   for (int l = cp->n_loop - 1; l >= 0; --l) {
     if (gp->mode == 2) {
-      VR_TIMED(ctx, "core_grow", s, k_cg_moments<<<(unsigned)K, kCT, 0, s>>>(
-          g.hoff, pre, g.u, g.v, gc, ex.searched, t, l, 0, 0.0));
+      VR_TIMED(ctx, "core_grow", s, k_cg_moments<<<(unsigned)(kCoreTeam * K), kCT, 0, s>>>(
+          g.hoff, pre, g.u, g.v, gc, ex.searched, t, l, hgrow, 0, 0.0));
       VR_LAUNCHED(ctx, "k_cg_moments");
     }
     VR_TIMED(ctx, "core_grow", s, k_cg_assign<<<grid_for(NHP, T), T, 0, s>>>(
