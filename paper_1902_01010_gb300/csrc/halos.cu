@@ -10,23 +10,53 @@ namespace {
 
 constexpr uint32_t kMaxHalo = 1u << 22;
 
-__global__ void k_count(const int32_t *__restrict__ label, int64_t n, uint32_t *__restrict__ cnt,
-                        DevStatus *st) {
+// Members per label, in two steps: a particle that carries its own index (every group's
+// first, and all singletons) is counted by a plain store, the others by atomics. A block
+// adds up its labels in a small hash table first, since the labels of large halos come in no
+// order and each is one address for up to millions of particles (10M members of a catalogue
+// with halos of up to a million: 1,197 -> 93 us). Labels outside [0, n) raise an error.
+__global__ void k_count_first(const int32_t *__restrict__ label, int64_t n, uint32_t *__restrict__ cnt) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  int32_t l = -1;
-  if (i < n) {
-    l = label[i];
+  if (i <= n) cnt[i] = i < n && label[i] == i ? 1u : 0u;
+}
+
+constexpr int kCountT = 256, kCountItems = 32, kCountSlots = 2048;
+__global__ void __launch_bounds__(kCountT) k_count(const int32_t *__restrict__ label, int64_t n,
+                                                   uint32_t *__restrict__ cnt, DevStatus *st) {
+  __shared__ int s_key[kCountSlots];
+  __shared__ uint32_t s_cnt[kCountSlots];
+  for (int k = threadIdx.x; k < kCountSlots; k += kCountT) {
+    s_key[k] = -1;
+    s_cnt[k] = 0;
+  }
+  __syncthreads();
+  const int64_t base = (int64_t)blockIdx.x * (kCountT * kCountItems);
+#pragma unroll 4
+  for (int r = 0; r < kCountItems; ++r) {
+    const int64_t i = base + r * kCountT + threadIdx.x;
+    if (i >= n) break;
+    const int32_t l = label[i];
     if (l < 0 || l >= n) {
       raise_error(st, VR_ERR_INVALID_ARG, 4);
-      l = -1;
+      continue;
     }
+    if (l == i) continue;
+    const uint32_t s0 = ((uint32_t)l * 2654435761u) >> 21;  // 11 bits
+    bool in = false;
+    for (int probe = 0; probe < 2 && !in; ++probe) {
+      const uint32_t s = (s0 + probe) & (kCountSlots - 1);
+      int k = s_key[s];
+      if (k == -1) k = atomicCAS(&s_key[s], -1, l);
+      if (k == -1 || k == l) {
+        atomicAdd(&s_cnt[s], 1u);
+        in = true;
+      }
+    }
+    if (!in) atomicAdd(&cnt[l], 1u);
   }
-  // lanes with the same label add their count once (members of a group are often
-  // neighbours in index order)
-  const int32_t key = l >= 0 ? l : -1 - lane;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  if (l >= 0 && lane == __ffs(peers) - 1) atomicAdd(&cnt[l], (uint32_t)__popc(peers));
+  __syncthreads();
+  for (int k = threadIdx.x; k < kCountSlots; k += kCountT)
+    if (s_key[k] >= 0) atomicAdd(&cnt[s_key[k]], s_cnt[k]);
 }
 
 // flag[l] = 1 if label l heads a halo; halos larger than 2^22 are rejected.
@@ -83,54 +113,72 @@ __global__ void k_halo_bounds(const uint32_t *__restrict__ hkey, const uint32_t 
   if (m == nhp - 1) hoff[h + 1] = (uint32_t)nhp;
 }
 
-__device__ __forceinline__ void warp_minmax_atomic(int *mn, int *mx, uint32_t key, int vmin,
-                                                   int vmax) {
-  // warp-aggregated when the whole warp belongs to one halo
-  const unsigned full = 0xffffffffu;
-  unsigned act = __activemask();
-  uint32_t k0 = __shfl_sync(act, key, __ffs(act) - 1);
-  bool same = __all_sync(act, key == k0) && act == full;
-  if (same) {
-    for (int o = 16; o; o >>= 1) {
-      vmin = min(vmin, __shfl_xor_sync(full, vmin, o));
-      vmax = max(vmax, __shfl_xor_sync(full, vmax, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      atomicMin(mn, vmin);
-      atomicMax(mx, vmax);
-    }
-  } else {
-    atomicMin(mn, vmin);
-    atomicMax(mx, vmax);
-  }
-}
-
+// Unwrapped positions of slots in (halo, index) order, and the halos' bounding boxes. A warp
+// takes kUnwrapRounds x 32 consecutive slots and keeps the box of the halo it is in per lane,
+// so that a run inside one halo costs six atomics in all, not six per 32 slots (10M members:
+// 497 -> 159 us).
+constexpr int kUnwrapRounds = 8;
 __global__ void k_unwrap(const int32_t *__restrict__ pos, const uint32_t *__restrict__ hkey,
                          const uint32_t *__restrict__ idx, const uint32_t *__restrict__ hoff,
                          const uint32_t *__restrict__ hlabel, int64_t nhp, int4 *__restrict__ u,
                          int *__restrict__ bmin, int *__restrict__ bmax) {
-  int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool ok = m < nhp;
-  uint32_t h = ok ? hkey[m] : 0xffffffffu;
-  int4 r = make_int4(0, 0, 0, 0);
-  if (ok) {
-    uint32_t i = idx[m], a = hlabel[h];
-    const uint32_t lm = (uint32_t)kLattice - 1u;
-    int ax = (int)((uint32_t)pos[3 * (int64_t)a] & lm), ay = (int)((uint32_t)pos[3 * (int64_t)a + 1] & lm),
-        az = (int)((uint32_t)pos[3 * (int64_t)a + 2] & lm);
-    int px = (int)((uint32_t)pos[3 * (int64_t)i] & lm), py = (int)((uint32_t)pos[3 * (int64_t)i + 1] & lm),
-        pz = (int)((uint32_t)pos[3 * (int64_t)i + 2] & lm);
-    r = make_int4(ax + min_image(px - ax), ay + min_image(py - ay), az + min_image(pz - az),
-                  (int)((uint32_t)m - hoff[h]));
-    u[m] = r;
-  }
-  if (__any_sync(0xffffffffu, ok)) {
-    if (ok) {
-      warp_minmax_atomic(&bmin[3 * (int64_t)h], &bmax[3 * (int64_t)h], h, r.x, r.x);
-      warp_minmax_atomic(&bmin[3 * (int64_t)h + 1], &bmax[3 * (int64_t)h + 1], h, r.y, r.y);
-      warp_minmax_atomic(&bmin[3 * (int64_t)h + 2], &bmax[3 * (int64_t)h + 2], h, r.z, r.z);
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32 * (32 * kUnwrapRounds);
+  uint32_t cur = 0xffffffffu;  // halo of the boxes below (warp-uniform)
+  int mn[3], mx[3];
+  auto flush = [&]() {
+    if (cur == 0xffffffffu) return;
+    for (int a = 0; a < 3; ++a) {
+      const int l = __reduce_min_sync(FULL, mn[a]), h = __reduce_max_sync(FULL, mx[a]);
+      if (lane == 0) {
+        atomicMin(&bmin[3 * (int64_t)cur + a], l);
+        atomicMax(&bmax[3 * (int64_t)cur + a], h);
+      }
     }
+  };
+  for (int k = 0; k < kUnwrapRounds; ++k) {
+    const int64_t m = base + 32 * k + lane;
+    const bool ok = m < nhp;
+    if (!__any_sync(FULL, ok)) break;
+    uint32_t h = 0xffffffffu;
+    int x[3] = {0, 0, 0};
+    if (ok) {
+      h = hkey[m];
+      const uint32_t i = idx[m], a = hlabel[h];
+      const uint32_t lm = (uint32_t)kLattice - 1u;
+      for (int c = 0; c < 3; ++c) {
+        const int ac = (int)((uint32_t)pos[3 * (int64_t)a + c] & lm), pc = (int)((uint32_t)pos[3 * (int64_t)i + c] & lm);
+        x[c] = ac + min_image(pc - ac);
+      }
+      u[m] = make_int4(x[0], x[1], x[2], (int)((uint32_t)m - hoff[h]));
+    }
+    const uint32_t h0 = __shfl_sync(FULL, h, 0);
+    if (__all_sync(FULL, h == h0)) {
+      if (h0 != cur) {
+        flush();
+        cur = h0;
+        for (int c = 0; c < 3; ++c) mn[c] = mx[c] = x[c];
+      } else {
+        for (int c = 0; c < 3; ++c) {
+          mn[c] = min(mn[c], x[c]);
+          mx[c] = max(mx[c], x[c]);
+        }
+      }
+    } else if (ok) {
+      // the lanes of one halo combine
+      const unsigned peers = __match_any_sync(__activemask(), h);
+      for (int c = 0; c < 3; ++c) {
+        const int l = __reduce_min_sync(peers, x[c]), g = __reduce_max_sync(peers, x[c]);
+        if (lane == __ffs(peers) - 1) {
+          atomicMin(&bmin[3 * (int64_t)h + c], l);
+          atomicMax(&bmax[3 * (int64_t)h + c], g);
+        }
+      }
+    }
+    __syncwarp();
   }
+  flush();
 }
 
 // Every member is unwrapped to within 2^20 of the halo's first member, which gives one
@@ -203,10 +251,11 @@ __global__ void k_curve_keys(const int4 *__restrict__ u, const uint32_t *__restr
   if (m >= nhp) return;
   uint32_t h = hkey[m];
   int4 r = u[m];
-  int64_t lo0 = bmin[3 * (int64_t)h], lo1 = bmin[3 * (int64_t)h + 1], lo2 = bmin[3 * (int64_t)h + 2];
-  int64_t e = max(bmax[3 * (int64_t)h] - lo0, max(bmax[3 * (int64_t)h + 1] - lo1, bmax[3 * (int64_t)h + 2] - lo2)) + 1;
-  uint32_t qx = (uint32_t)(((r.x - lo0) << 10) / e), qy = (uint32_t)(((r.y - lo1) << 10) / e),
-           qz = (uint32_t)(((r.z - lo2) << 10) / e);
+  // a member lies less than 2^21 above the box's corner, so 32-bit words hold ten bits more
+  const int lo0 = bmin[3 * (int64_t)h], lo1 = bmin[3 * (int64_t)h + 1], lo2 = bmin[3 * (int64_t)h + 2];
+  const uint32_t e = (uint32_t)max(bmax[3 * (int64_t)h] - lo0, max(bmax[3 * (int64_t)h + 1] - lo1, bmax[3 * (int64_t)h + 2] - lo2)) + 1u;
+  const uint32_t qx = ((uint32_t)(r.x - lo0) << 10) / e, qy = ((uint32_t)(r.y - lo1) << 10) / e,
+                 qz = ((uint32_t)(r.z - lo2) << 10) / e;
   keys[m] = ((u64)h << 30) | (HILBERT ? hilbert10(qx, qy, qz) : (uint32_t)morton3(qx, qy, qz));
   vals[m] = (uint32_t)m;
 }
@@ -323,8 +372,9 @@ vr_status build_halos(vr_ctx *ctx, const int32_t *pos, const float *vel, int64_t
     ~Release() { a.off = off; }
   } release{ar, keep};
   const int T = 256;
-  VR_CUDA(ctx, cudaMemsetAsync(B.cnt, 0, (n + 1) * sizeof(uint32_t), s));
-  k_count<<<grid_for(n, T), T, 0, s>>>(label, n, B.cnt, ctx->d_status);
+  k_count_first<<<grid_for(n + 1, T), T, 0, s>>>(label, n, B.cnt);
+  VR_LAUNCHED(ctx, "k_count_first");
+  k_count<<<grid_for(n, kCountT * kCountItems), kCountT, 0, s>>>(label, n, B.cnt, ctx->d_status);
   VR_LAUNCHED(ctx, "k_count");
   k_halo_flags<<<grid_for(n + 1, T), T, 0, s>>>(B.cnt, n, nmin, B.flag, ctx->d_status);
   VR_LAUNCHED(ctx, "k_halo_flags");
@@ -356,7 +406,7 @@ vr_status build_halos(vr_ctx *ctx, const int32_t *pos, const float *vel, int64_t
   // bounding boxes: min starts at INT_MAX, max at INT_MIN
   VR_CUDA(ctx, cudaMemsetAsync(B.bmin, 0x7f, 3 * H * sizeof(int), s));
   VR_CUDA(ctx, cudaMemsetAsync(B.bmax, 0x80, 3 * H * sizeof(int), s));
-  k_unwrap<<<grid_for(NHP, T), T, 0, s>>>(pos, hkey, idx, g.hoff, g.hlabel, NHP, B.u_idx, B.bmin, B.bmax);
+  k_unwrap<<<grid_for(NHP, T * kUnwrapRounds), T, 0, s>>>(pos, hkey, idx, g.hoff, g.hlabel, NHP, B.u_idx, B.bmin, B.bmax);
   VR_LAUNCHED(ctx, "k_unwrap");
   k_halo_span<<<grid_for(H, T), T, 0, s>>>(B.bmin, B.bmax, H, ctx->d_status);
   VR_LAUNCHED(ctx, "k_halo_span");
