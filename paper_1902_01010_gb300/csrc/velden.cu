@@ -7,11 +7,11 @@
 //    buckets of one halo form a "super-bucket";
 //  - one warp handles one bucket: lane k is the query particle k. Each lane first bounds
 //    its N_se-th neighbour distance by the N_se-th smallest distance among the 4 N_se
-//    members around the bucket in Morton order (to within one of 32 histogram bins);
+//    members around the bucket in Morton order (to within one of 64 histogram bins);
 //    every later pass visits only the buckets whose boxes come within the largest
 //    per-lane bound of the warp's own box (super-bucket boxes prune first);
 //  - each visited bucket is staged once in shared memory and read back by every lane
-//    with broadcast 16-byte loads; every lane keeps its own 32-bin histogram of the exact
+//    with broadcast 16-byte loads; every lane keeps its own 64-bin histogram of the exact
 //    key (d^2 << 22 | local index). Histogram passes narrow the key range until the bin
 //    holding the N_se-th key has at most 16 keys; a last pass feeds every key below that
 //    bin, plus the right number from the bin, into a per-lane list of the N_v smallest
@@ -21,7 +21,11 @@
 // Position keys are exact integers, so the N_se set equals the oracle's; velocity
 // differences and sums are FP32. Squared separations are 64-bit integers, or 32-bit ones
 // wherever the two boxes involved (query bucket and candidate bucket or window) bound
-// every separation by 32767 lattice units per axis, which makes them exact in uint32.
+// every separation by kNarrow lattice units per axis, which makes them exact in 32 bits.
+//
+// What bounds the pass over a 256^3 box (51.9 ms): the issue of the window's and the levels'
+// members (30 ms), the visits of the collect pass (9), the list insertions, whose lanes
+// diverge (6), the keys of the final bin (4) and the halos' layout (2).
 // Halos with at most N_se members use every member (one pass, no position search).
 #include <math.h>
 
@@ -53,16 +57,19 @@ constexpr int kStatPass0 = 1;    // info[1 + pass]: 0 window, 1.. histogram leve
 constexpr int kWindow = 4;       // window of kWindow * N_se members for the first bound
 
 // Per-warp shared memory. The key histogram is used only by the bound and histogram
-// passes and the final-bin buffer only by the collect pass, so the two share storage.
+// passes and the top-N_v list only by the collect pass, so the two share storage and the
+// slots of the final bin are in local memory (5 KB a warp; with the list in a storage of its own,
+// beside counts that shared with the slots, it was 9 KB: f_l of a 256^3 box 57.9 ms, 54.3 so).
+// Counts of 32 bits, a bank per lane, were tried: 52.4 ms with shared-memory atomics and 54.0
+// with plain loads and stores, against 51.9 for 16 bits.
 template <int NVM>
 struct WarpSmem {
   int4 su[32];
   float4 sv[32];
   union {
-    uint16_t hist[kBins][32];
-    uint32_t bslot[kBuf][32];  // member slots of the keys in the final bin
+    uint16_t hist[kBins + 2][32];  // keys below the bins, the bins, keys beyond them
+    float top[NVM][32];
   };
-  float top[NVM][32];
 };
 
 template <int NVM>
@@ -142,22 +149,43 @@ __device__ __forceinline__ long long d2i(int4 a, int4 b) {
   long long dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
   return dx * dx + dy * dy + dz * dz;
 }
-// The same squared separation in 32-bit arithmetic, exact when every component of a - b
-// lies in [-32767, 32767]: then d^2 < 3 * 2^30 < 2^32.
-__device__ __forceinline__ uint32_t d2u(int4 a, int4 b) {
-  const int dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-  return (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
+// The 32-bit route. When the query box is at most kNarrow wide and every separation between a
+// point of it and one of the candidates' box has all components within kNarrow, d^2 < 2^31
+// and, with coordinates relative to the query box's corner o, |q|^2 < 2^31. Then d^2 =
+// |c|^2 - 2 q.c + |q|^2 in 32-bit arithmetic (what wraps on the way wraps back, and d^2 -
+// |q|^2 fits a signed word), so a candidate staged as (c, |c|^2) costs three multiply-adds,
+// and |q|^2 goes into the thresholds (f_l of a 256^3 box: 52.6 ms with three subtractions as
+// well, 51.9 so).
+constexpr int kNarrow = 26754;  // 3 kNarrow^2 < 2^31
+
+struct Rel {  // a query's side
+  uint32_t ax, ay, az;  // -2 (q - o)
+  int q2;               // |q - o|^2
+};
+__device__ __forceinline__ Rel rel_query(int4 q, int4 o) {
+  const uint32_t x = (uint32_t)(q.x - o.x), y = (uint32_t)(q.y - o.y), z = (uint32_t)(q.z - o.z);
+  return Rel{0u - 2u * x, 0u - 2u * y, 0u - 2u * z, (int)(x * x + y * y + z * z)};
+}
+__device__ __forceinline__ int4 rel_member(int4 p, int4 o) {
+  const uint32_t x = (uint32_t)(p.x - o.x), y = (uint32_t)(p.y - o.y), z = (uint32_t)(p.z - o.z);
+  return make_int4((int)x, (int)y, (int)z, (int)(x * x + y * y + z * z));
+}
+// d^2 - |q - o|^2
+__device__ __forceinline__ int rel_d2(const Rel &r, int4 c) {
+  return (int)(r.ax * (uint32_t)c.x + (r.ay * (uint32_t)c.y + (r.az * (uint32_t)c.z + (uint32_t)c.w)));
 }
 
-// True when every separation between a point of box A and a point of box B has all
-// components in [-32767, 32767] (d2u is then exact for every such pair).
+// True when the query box A is at most kNarrow wide and every separation between a point of
+// it and a point of box B has all components within kNarrow.
 __device__ __forceinline__ bool fits32(int4 alo, int4 ahi, int4 blo, int4 bhi) {
-  const int ex = max(ahi.x - blo.x, bhi.x - alo.x), ey = max(ahi.y - blo.y, bhi.y - alo.y),
-            ez = max(ahi.z - blo.z, bhi.z - alo.z);
-  return max(ex, max(ey, ez)) <= 32767;
+  const int ex = max(ahi.x - min(alo.x, blo.x), bhi.x - alo.x),
+            ey = max(ahi.y - min(alo.y, blo.y), bhi.y - alo.y),
+            ez = max(ahi.z - min(alo.z, blo.z), bhi.z - alo.z);
+  return max(ex, max(ey, ez)) <= kNarrow;
 }
 
-__device__ __forceinline__ uint32_t clamp32(u64 x) { return x > 0xffffffffull ? 0xffffffffu : (uint32_t)x; }
+// A bound on d^2 for the 32-bit route, where d^2 < 2^31.
+__device__ __forceinline__ int clamp31(u64 x) { return x > 0x7fffffffull ? 0x7fffffff : (int)x; }
 
 // ---------------------------------------------------------------- small halos
 // Halos of at most N_se members: every member is a neighbour. A warp takes 32 consecutive
@@ -346,9 +374,16 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
   // stages slots [s0, s0 + cnt) in shared memory (positions; velocities if asked); the
   // remaining entries get a sentinel position far outside any bound (d^2 > 2^58), so the
   // candidate loops always run 32 fixed iterations
-  auto stage = [&](uint32_t s0, int cnt, bool with_v) {
+  // (`rel`: relative to the query box's corner, for the 32-bit route)
+  const int4 qlo = bmin[b], qhi = bmax[b];
+  const Rel rq = rel_query(q, qlo);
+  auto stage = [&](uint32_t s0, int cnt, bool with_v, bool rel) {
     __syncwarp();
-    if (lane < cnt) {
+    if (rel) {  // beyond `cnt`: the last one again
+      const uint32_t m = s0 + min(lane, cnt - 1);
+      sm.su[lane] = rel_member(u[m], qlo);
+      if (with_v) sm.sv[lane] = v[m];
+    } else if (lane < cnt) {
       sm.su[lane] = u[s0 + lane];
       if (with_v) sm.sv[lane] = v[s0 + lane];
     } else {
@@ -357,10 +392,9 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     __syncwarp();
     VR_STAT(st, kStatPass0 + pass_id, 1);
   };
-  const int4 qlo = bmin[b], qhi = bmax[b];
   // 1. bound from the window of kWindow * N_se members around the bucket: the N_se-th
   //    smallest distance among them, rounded up to a histogram bin edge. When the window's
-  //    box and the bucket's box bound every separation by 32767 per axis (a warp-uniform
+  //    box and the bucket's box bound every separation by kNarrow per axis (a warp-uniform
   //    test), the distances are exact in 32-bit arithmetic.
   long long r2 = 0;
   {
@@ -385,17 +419,14 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     }
     const bool wn = fits32(qlo, qhi, wlo, whi);  // warp-uniform
     long long wmax = 0;
-    uint32_t wmax32 = 0;
+    int wmax32 = -0x7fffffff;  // of d^2 - |q - o|^2
     for (int c = 0; c < W; c += 32) {
       const int cnt = min(32, W - c);
-      stage((uint32_t)(w0 + c), cnt, false);
+      stage((uint32_t)(w0 + c), cnt, false, wn);
       if (wn) {
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
-          uint32_t d[BATCH];
 #pragma unroll
-          for (int j = 0; j < BATCH; ++j) d[j] = d2u(q, sm.su[t0 + j]);
-#pragma unroll
-          for (int j = 0; j < BATCH; ++j) wmax32 = (t0 + j < cnt && d[j] > wmax32) ? d[j] : wmax32;
+          for (int j = 0; j < BATCH; ++j) wmax32 = max(wmax32, rel_d2(rq, sm.su[t0 + j]));
         }
       } else {
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
@@ -407,22 +438,22 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
         }
       }
     }
-    if (wn) wmax = (long long)wmax32;
+    if (wn) wmax = (long long)wmax32 + rq.q2;
     for (int cb = 0; cb < kBins; ++cb) sm.hist[cb][lane] = 0;
     int sh0 = bitlen64((unsigned long long)wmax) - kBinBits;  // kBins bins over [0, 2^bitlen)
     if (sh0 < 0) sh0 = 0;
     for (int c = 0; c < W; c += 32) {
       const int cnt = min(32, W - c);
-      stage((uint32_t)(w0 + c), cnt, false);
-      if (wn) {  // wmax < 2^32, so sh0 <= 26
+      stage((uint32_t)(w0 + c), cnt, false, wn);
+      if (wn) {  // wmax < 2^31, so sh0 <= 25
+        int d[BATCH];
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
-          uint32_t d[BATCH];
 #pragma unroll
-          for (int j = 0; j < BATCH; ++j) d[j] = d2u(q, sm.su[t0 + j]);
+          for (int j = 0; j < BATCH; ++j) d[j] = rel_d2(rq, sm.su[t0 + j]) + rq.q2;
 #pragma unroll
-          for (int j = 0; j < BATCH; ++j)
-            if (t0 + j < cnt) sm.hist[d[j] >> sh0][lane]++;
+          for (int j = 0; j < BATCH; ++j) sm.hist[d[j] >> sh0][lane]++;
         }
+        sm.hist[d[BATCH - 1] >> sh0][lane] -= 32 - cnt;  // the repeated last one
       } else {
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
           long long d[BATCH];
@@ -485,37 +516,42 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
   bool focus = true;    // this lane's current level is the focused first level
   for (int level = 0; level < 16; ++level) {
     pass_id = level < 5 ? 1 + level : 5;
-    int below = 0;
+    int below = 0, seen = 0;
     if (!settled)
-      for (int c = 0; c < kBins; ++c) sm.hist[c][lane] = 0;
+      for (int c = 0; c < kBins + 2; ++c) sm.hist[c][lane] = 0;
     const long long rmax2 = warp_max(settled ? -1 : rcur);
     for_each_bucket(rmax2, [&](uint32_t bb) {
       bool want = !settled && pt_box_d2(q, bmin[bb], bmax[bb]) <= rcur;
       if (!__any_sync(FULL, want)) return;
       const uint32_t s0 = hs + 32u * (bb - 32u * sb0);
       const int cnt = (int)min(32u, he - s0);
-      stage(s0, cnt, false);
-      // 32-bit route: the boxes bound every separation by 32767 per axis and the bins
-      // are at least one unit of d^2 wide, so a key's bin depends on d^2 alone (klo is a
-      // multiple of 2^22): bin = (d^2 - (klo >> 22)) >> (sh - 22)
-      const bool narrow = fits32(qlo, qhi, bmin[bb], bmax[bb]);
-      if (want && narrow && sh >= 22 && (klo & 0x3fffffull) == 0) {
-        const uint32_t r32 = clamp32((u64)rcur), dlo = clamp32(klo >> 22);
-        const int shd = sh - 22;
+      // 32-bit route: the boxes are near enough and the bins of every lane are whole units of
+      // d^2, so a key's bin depends on d^2 alone (klo is a multiple of 2^22): bin =
+      // (d^2 - (klo >> 22)) >> (sh - 22)
+      const bool narrow = fits32(qlo, qhi, bmin[bb], bmax[bb]) &&
+                          __all_sync(FULL, !want || (sh >= 22 && sh < 53 && (klo & 0x3fffffull) == 0));
+      stage(s0, cnt, false, narrow);
+      if (narrow) {
+        // without a branch per member: what lies below the bins or beyond the bound (all of it
+        // for a lane that wants none) counts in a row of its own (f_l of a 256^3 box: 54.3 ms
+        // with a compare and a branch for each, 51.8 so)
+        const int far = (want ? clamp31((u64)rcur) : -1) - rq.q2, off = rq.q2 - clamp31(klo >> 22);
+        const int shd = want ? sh - 22 : 0;
+        auto row_of = [&](int x) { return x > far ? kBins + 1 : max((x + off) >> shd, -1) + 1; };
+        int d[BATCH];
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
-          uint32_t d[BATCH];
 #pragma unroll
-          for (int j = 0; j < BATCH; ++j) d[j] = d2u(q, sm.su[t0 + j]);
+          for (int j = 0; j < BATCH; ++j) d[j] = rel_d2(rq, sm.su[t0 + j]);
 #pragma unroll
-          for (int j = 0; j < BATCH; ++j) {
-            if (t0 + j < cnt && d[j] <= r32) {
-              if (d[j] >= dlo) {
-                const uint32_t rel = shd >= 32 ? 0u : (d[j] - dlo) >> shd;
-                if (rel < kBins) sm.hist[rel][lane]++;
-              } else if (focus) {
-                ++below;
-              }
-            }
+          for (int j = 0; j < BATCH; ++j) sm.hist[row_of(d[j])][lane]++;
+        }
+        sm.hist[row_of(d[BATCH - 1])][lane] -= 32 - cnt;  // the repeated last one
+        seen += 32;
+        if (seen > 0xffff - 32) {  // before the 16-bit count of row 0 could wrap
+          seen = 0;
+          if (!settled) {
+            below += sm.hist[0][lane];
+            sm.hist[0][lane] = 0;
           }
         }
       } else if (want) {
@@ -529,7 +565,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
               u64 key = ((u64)d[j] << 22) | (u64)sm.su[t0 + j].w;
               if (key >= klo) {
                 u64 rel = (key - klo) >> sh;
-                if (rel < kBins) sm.hist[rel][lane]++;
+                if (rel < kBins) sm.hist[1 + rel][lane]++;
               } else if (focus) {
                 ++below;
               }
@@ -539,6 +575,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       }
     });
     if (!settled) {
+      below += sm.hist[0][lane];
       if (focus && below >= need) {
         // the N_se-th key lies below the focused range: bin [0, klo) next
         const u64 hi = klo;
@@ -553,14 +590,14 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
         focus = false;
         int cum = 0, bs = kBins - 1;
         for (int c = 0; c < kBins; ++c) {
-          int hc = sm.hist[c][lane];
+          int hc = sm.hist[1 + c][lane];
           if (cum + hc >= need) {
             bs = c;
             break;
           }
           cum += hc;
         }
-        int hc = sm.hist[bs][lane];
+        int hc = sm.hist[1 + bs][lane];
         if (hc <= kBuf || sh == 0) {
           fin_lo = klo + ((u64)bs << sh);
           fin_hi = fin_lo + ((u64)1 << sh);
@@ -587,37 +624,39 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
   float(*top)[32] = sm.top;
   TopV tv = {0, 0, 0.0f};
   int nbuf = 0;
+  uint32_t bslot[kBuf];  // member slots of the keys in the final bin (a few, in local memory)
   pass_id = 6;
   for_each_bucket(warp_max(rcur), [&](uint32_t bb) {
     bool want = valid && pt_box_d2(q, bmin[bb], bmax[bb]) <= rcur;
     if (!__any_sync(FULL, want)) return;
     const uint32_t s0 = hs + 32u * (bb - 32u * sb0);
     const int cnt = (int)min(32u, he - s0);
-    stage(s0, cnt, true);
     // 32-bit route as in the histogram passes: with both final-bin edges multiples of
     // 2^22, key < edge iff d^2 < edge >> 22
-    const bool narrow = fits32(qlo, qhi, bmin[bb], bmax[bb]);
-    if (want && narrow && ((fin_lo | fin_hi) & 0x3fffffull) == 0) {
-      const uint32_t r32 = clamp32((u64)rcur), flo = clamp32(fin_lo >> 22),
-                     fhi = clamp32(fin_hi >> 22);
+    const bool narrow = fits32(qlo, qhi, bmin[bb], bmax[bb]) &&
+                        __all_sync(FULL, !want || ((fin_lo | fin_hi) & 0x3fffffull) == 0);
+    stage(s0, cnt, true, narrow);
+    if (narrow && want) {
+      const int far = (want ? clamp31((u64)rcur) : -1) - rq.q2, flo = clamp31(fin_lo >> 22) - rq.q2,
+                fhi = clamp31(fin_hi >> 22) - rq.q2;
       for (int t0 = 0; t0 < 32; t0 += BATCH) {
-        uint32_t d[BATCH];
+        int d[BATCH];
 #pragma unroll
-        for (int j = 0; j < BATCH; ++j) d[j] = d2u(q, sm.su[t0 + j]);
+        for (int j = 0; j < BATCH; ++j) d[j] = rel_d2(rq, sm.su[t0 + j]);
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) {
-          if (t0 + j < cnt && d[j] <= r32) {
+          if (t0 + j < cnt && d[j] <= far) {
             const int t = t0 + j;
             if (d[j] < flo) {
               top_insert(top, lane, tv, nv_eff, dv2f(sm.sv[t], vq));
             } else if (d[j] < fhi && nbuf < kBuf) {
-              sm.bslot[nbuf][lane] = s0 + (uint32_t)t;
+              bslot[nbuf] = s0 + (uint32_t)t;
               ++nbuf;
             }
           }
         }
       }
-    } else if (want) {
+    } else if (want && !narrow) {
       for (int t0 = 0; t0 < 32; t0 += BATCH) {
         long long d[BATCH];
 #pragma unroll
@@ -630,7 +669,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
             if (key < fin_lo) {
               top_insert(top, lane, tv, nv_eff, dv2f(sm.sv[t], vq));
             } else if (key < fin_hi && nbuf < kBuf) {
-              sm.bslot[nbuf][lane] = s0 + (uint32_t)t;
+              bslot[nbuf] = s0 + (uint32_t)t;
               ++nbuf;
             }
           }
@@ -645,7 +684,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     int best = -1;
     u64 bk = ~0ULL;
     for (int e = 0; e < nbuf; ++e) {
-      const int4 pe = u[sm.bslot[e][lane]];
+      const int4 pe = u[bslot[e]];
       const u64 x = ((u64)d2i(q, pe) << 22) | (u64)pe.w;
       if ((r == 0 || x > last) && x < bk) {
         bk = x;
@@ -654,7 +693,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     }
     if (best < 0) break;
     last = bk;
-    top_insert(top, lane, tv, nv_eff, dv2f(v[sm.bslot[best][lane]], vq));
+    top_insert(top, lane, tv, nv_eff, dv2f(v[bslot[best]], vq));
   }
   f_l[__float_as_int(vq.w)] = top_density(top, lane, tv, nse_eff);
 }
