@@ -15,7 +15,7 @@ struct VShape {
   int batch, maxreg, warps;
 };
 constexpr int kNVShapes = 5;
-constexpr VShape kVShapes[kNVShapes] = {{4, 80, 4}, {4, 80, 8}, {4, 80, 2}, {2, 80, 4}, {8, 96, 4}};
+constexpr VShape kVShapes[kNVShapes] = {{4, 64, 4}, {4, 64, 8}, {4, 64, 2}, {2, 64, 4}, {8, 80, 4}};
 
 // 6D linker shapes: warps (32-candidate tiles) per block.
 constexpr int kNLShapes = 3;

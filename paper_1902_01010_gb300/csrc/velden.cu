@@ -23,9 +23,11 @@
 // wherever the two boxes involved (query bucket and candidate bucket or window) bound
 // every separation by kNarrow lattice units per axis, which makes them exact in 32 bits.
 //
-// What bounds the pass over a 256^3 box (51.9 ms): the issue of the window's and the levels'
-// members (30 ms), the visits of the collect pass (9), the list insertions, whose lanes
-// diverge (6), the keys of the final bin (4) and the halos' layout (2).
+// What bounds the pass over a 256^3 box (36 ms): the issue slots (71 % taken at 5 warps a
+// scheduler), by phase the window's bound 7 %, the histogram levels 38 %, the collect pass 42 %
+// (most of it list insertions, whose lanes diverge), the keys of the final bin 13 %. Its code has
+// to stay small: with every loop over 32 members unrolled whole, warps in different phases put
+// each other's instructions out of the cache, and the same work took 44.6 ms instead of 39.4.
 // Halos with at most N_se members use every member (one pass, no position search).
 #include <math.h>
 
@@ -70,6 +72,8 @@ struct WarpSmem {
     uint16_t hist[kBins + 2][32];  // keys below the bins, the bins, keys beyond them
     float top[NVM][32];
   };
+  int4 blo[32], bhi[32];  // boxes of 32 candidate buckets
+  int4 qlo[2], qhi[2];    // boxes of the query bucket's two parts
 };
 
 template <int NVM>
@@ -424,11 +428,13 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       const int cnt = min(32, W - c);
       stage((uint32_t)(w0 + c), cnt, false, wn);
       if (wn) {
+#pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
 #pragma unroll
           for (int j = 0; j < BATCH; ++j) wmax32 = max(wmax32, rel_d2(rq, sm.su[t0 + j]));
         }
       } else {
+#pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
           long long d[BATCH];
 #pragma unroll
@@ -439,6 +445,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       }
     }
     if (wn) wmax = (long long)wmax32 + rq.q2;
+#pragma unroll 4
     for (int cb = 0; cb < kBins; ++cb) sm.hist[cb][lane] = 0;
     int sh0 = bitlen64((unsigned long long)wmax) - kBinBits;  // kBins bins over [0, 2^bitlen)
     if (sh0 < 0) sh0 = 0;
@@ -447,6 +454,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       stage((uint32_t)(w0 + c), cnt, false, wn);
       if (wn) {  // wmax < 2^31, so sh0 <= 25
         int d[BATCH];
+#pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
 #pragma unroll
           for (int j = 0; j < BATCH; ++j) d[j] = rel_d2(rq, sm.su[t0 + j]) + rq.q2;
@@ -455,6 +463,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
         }
         sm.hist[d[BATCH - 1] >> sh0][lane] -= 32 - cnt;  // the repeated last one
       } else {
+#pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
           long long d[BATCH];
 #pragma unroll
@@ -466,6 +475,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       }
     }
     int cum = 0, bs = kBins - 1;
+#pragma unroll 4
     for (int cb = 0; cb < kBins; ++cb) {
       cum += sm.hist[cb][lane];
       if (cum >= nse_eff) {
@@ -480,25 +490,102 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     raise_error(st, VR_ERR_UNSUPPORTED, 1);
     return;
   }
+  // Two parts of the query bucket: where the curve jumps, its particles lie in two clumps, and
+  // one box would reach everything between them (in a halo of 564 k members one bucket
+  // tested 27,000 others one by one for 437 to visit: 25 M cycles, 13 ms, as long as the launch's
+  // other warps together; with two parts 6 M).
+  // Boxes of the particles up to each lane and from each lane on; the cut is where the two
+  // volumes are least, each extent with an eighth of the largest one added.
+  int cut = 31;
+  {
+    int4 alo = q, ahi = q, zlo = q, zhi = q;  // lanes beyond the bucket repeat its first particle
+    const int last = (int)(qe - qs) - 1;
+    auto from = [&](int4 a, int src) {
+      return make_int4(__shfl_sync(FULL, a.x, src), __shfl_sync(FULL, a.y, src), __shfl_sync(FULL, a.z, src), 0);
+    };
+    auto join = [](int4 &lo, int4 &hi, int4 l, int4 h) {
+      lo.x = min(lo.x, l.x); lo.y = min(lo.y, l.y); lo.z = min(lo.z, l.z);
+      hi.x = max(hi.x, h.x); hi.y = max(hi.y, h.y); hi.z = max(hi.z, h.z);
+    };
+    for (int o = 1; o < 32; o <<= 1) {
+      const int4 al = from(alo, lane - o), ah = from(ahi, lane - o), zl = from(zlo, lane + o), zh = from(zhi, lane + o);
+      if (lane >= o) join(alo, ahi, al, ah);
+      if (lane + o <= last) join(zlo, zhi, zl, zh);
+    }
+    const float m = 0.125f * (float)max(qhi.x - qlo.x, max(qhi.y - qlo.y, qhi.z - qlo.z));
+    auto vol = [&](int4 l, int4 h) {
+      return ((float)(h.x - l.x) + m) * ((float)(h.y - l.y) + m) * ((float)(h.z - l.z) + m);
+    };
+    const int4 nlo = from(zlo, lane + 1), nhi = from(zhi, lane + 1);
+    float best = lane < last ? vol(alo, ahi) + vol(nlo, nhi) : __int_as_float(0x7f800000);
+    int at = lane;
+    for (int o = 16; o; o >>= 1) {
+      const float ob = __shfl_xor_sync(FULL, best, o);
+      const int oa = __shfl_xor_sync(FULL, at, o);
+      if (ob < best || (ob == best && oa < at)) {
+        best = ob;
+        at = oa;
+      }
+    }
+    cut = at;  // 0 for a single particle, whose second part has no lane that wants anything
+    if (lane == at) {
+      sm.qlo[0] = alo;
+      sm.qhi[0] = ahi;
+      sm.qlo[1] = last > 0 ? nlo : alo;
+      sm.qhi[1] = last > 0 ? nhi : ahi;
+    }
+    __syncwarp();
+  }
   // Candidate buckets are enumerated on the fly in every pass: super-bucket boxes, then
   // bucket boxes, against the query bucket's box grown by the largest per-lane bound;
   // f(bucket index) is called warp-uniformly for every bucket that passes.
-  auto for_each_bucket = [&](long long rmax2, auto &&f) {
+  // f(bucket index, this lane wants it, it fits the 32-bit route) returns true when it lowered
+  // a lane's bound.
+  auto for_each_bucket = [&](const long long &r2lane, auto &&f) {
+    long long ra, rz;  // largest bounds in the query bucket's parts
+    auto bounds = [&]() {
+      ra = warp_max(lane <= cut ? r2lane : -1);
+      rz = warp_max(lane <= cut ? -1 : r2lane);
+    };
+    auto reach = [&](int4 lo, int4 hi) {
+      return box_d2(sm.qlo[0], sm.qhi[0], lo, hi) <= ra || box_d2(sm.qlo[1], sm.qhi[1], lo, hi) <= rz;
+    };
+    auto gap = [](int lo, int hi, int c) { return max(max(lo - c, c - hi), 0); };
+    bounds();
     for (uint32_t sbase = sb0; sbase < sb1; sbase += 32) {
       uint32_t sx = sbase + lane;
-      bool hit = sx < sb1 && box_d2(qlo, qhi, smin[sx], smax[sx]) <= rmax2;
+      bool hit = sx < sb1 && reach(smin[sx], smax[sx]);
       unsigned hm = __ballot_sync(FULL, hit);
       while (hm) {
         int t = __ffs(hm) - 1;
         hm &= hm - 1;
-        uint32_t bb = 32u * (sbase + t) + lane;
-        bool in = (bb - 32u * sb0) < nbh && box_d2(qlo, qhi, bmin[bb], bmax[bb]) <= rmax2;
-        unsigned bm = __ballot_sync(FULL, in);
-        while (bm) {
-          int tb = __ffs(bm) - 1;
-          bm &= bm - 1;
-          f(32u * (sbase + t) + (uint32_t)tb);
+        const uint32_t bb = 32u * (sbase + t) + lane;
+        bool in = false, near = false;
+        if (bb - 32u * sb0 < nbh) {
+          const int4 lo = bmin[bb], hi = bmax[bb];
+          in = reach(lo, hi);
+          near = fits32(qlo, qhi, lo, hi);
+          sm.blo[lane] = lo;
+          sm.bhi[lane] = hi;
         }
+        unsigned bm = __ballot_sync(FULL, in);
+        const unsigned nm = __ballot_sync(FULL, near);
+        __syncwarp();
+        while (bm) {
+          const int tb = __ffs(bm) - 1;
+          bm &= bm - 1;
+          const bool fits = (nm >> tb) & 1u;
+          const int4 lo = sm.blo[tb], hi = sm.bhi[tb];
+          bool want;
+          if (fits) {
+            const int ax = gap(lo.x, hi.x, q.x), ay = gap(lo.y, hi.y, q.y), az = gap(lo.z, hi.z, q.z);
+            want = ax * ax + ay * ay + az * az <= (r2lane < 0 ? -1 : clamp31((u64)r2lane));
+          } else {
+            want = pt_box_d2(q, lo, hi) <= r2lane;
+          }
+          if (__any_sync(FULL, want) && f(32u * (sbase + t) + (uint32_t)tb, want, fits)) bounds();
+        }
+        __syncwarp();
       }
     }
   };
@@ -516,29 +603,28 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
   bool focus = true;    // this lane's current level is the focused first level
   for (int level = 0; level < 16; ++level) {
     pass_id = level < 5 ? 1 + level : 5;
-    int below = 0, seen = 0;
+    int below = 0, seen = 0, visits = 0;
+    long long rlev = settled ? -1 : rcur;  // bound on d^2 of the keys that this level has to count
     if (!settled)
+#pragma unroll 4
       for (int c = 0; c < kBins + 2; ++c) sm.hist[c][lane] = 0;
-    const long long rmax2 = warp_max(settled ? -1 : rcur);
-    for_each_bucket(rmax2, [&](uint32_t bb) {
-      bool want = !settled && pt_box_d2(q, bmin[bb], bmax[bb]) <= rcur;
-      if (!__any_sync(FULL, want)) return;
+    for_each_bucket(rlev, [&](uint32_t bb, bool want, bool fits) {
       const uint32_t s0 = hs + 32u * (bb - 32u * sb0);
       const int cnt = (int)min(32u, he - s0);
       // 32-bit route: the boxes are near enough and the bins of every lane are whole units of
       // d^2, so a key's bin depends on d^2 alone (klo is a multiple of 2^22): bin =
       // (d^2 - (klo >> 22)) >> (sh - 22)
-      const bool narrow = fits32(qlo, qhi, bmin[bb], bmax[bb]) &&
-                          __all_sync(FULL, !want || (sh >= 22 && sh < 53 && (klo & 0x3fffffull) == 0));
+      const bool narrow = fits && __all_sync(FULL, !want || (sh >= 22 && sh < 53 && (klo & 0x3fffffull) == 0));
       stage(s0, cnt, false, narrow);
       if (narrow) {
         // without a branch per member: what lies below the bins or beyond the bound (all of it
         // for a lane that wants none) counts in a row of its own (f_l of a 256^3 box: 54.3 ms
         // with a compare and a branch for each, 51.8 so)
-        const int far = (want ? clamp31((u64)rcur) : -1) - rq.q2, off = rq.q2 - clamp31(klo >> 22);
+        const int far = (want ? clamp31((u64)rlev) : -1) - rq.q2, off = rq.q2 - clamp31(klo >> 22);
         const int shd = want ? sh - 22 : 0;
         auto row_of = [&](int x) { return x > far ? kBins + 1 : max((x + off) >> shd, -1) + 1; };
         int d[BATCH];
+#pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
 #pragma unroll
           for (int j = 0; j < BATCH; ++j) d[j] = rel_d2(rq, sm.su[t0 + j]);
@@ -555,13 +641,14 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
           }
         }
       } else if (want) {
+#pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
           long long d[BATCH];
 #pragma unroll
           for (int j = 0; j < BATCH; ++j) d[j] = d2i(q, sm.su[t0 + j]);
 #pragma unroll
           for (int j = 0; j < BATCH; ++j) {
-            if (d[j] <= rcur) {
+            if (d[j] <= rlev) {
               u64 key = ((u64)d[j] << 22) | (u64)sm.su[t0 + j].w;
               if (key >= klo) {
                 u64 rel = (key - klo) >> sh;
@@ -573,6 +660,27 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
           }
         }
       }
+      // Every 32 buckets: the bins counted so far bound the N_se-th key already, and nothing beyond
+      // the bin that reaches it matters.
+      if (++visits & 31) return false;
+      if (rlev >= 0) {
+        int cum = below + (int)sm.hist[0][lane];
+        if (!focus) cum = 0;
+        if (cum >= need) {
+          rlev = -1;  // it lies below the focused range: nothing more to count here
+        } else {
+#pragma unroll 4
+          for (int c = 0; c < kBins; ++c) {
+            cum += sm.hist[1 + c][lane];
+            if (cum >= need) {
+              const long long top_d = (long long)((klo + ((u64)(c + 1) << sh) - 1) >> 22);
+              rlev = top_d < rlev ? top_d : rlev;
+              break;
+            }
+          }
+        }
+      }
+      return true;
     });
     if (!settled) {
       below += sm.hist[0][lane];
@@ -589,6 +697,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
         if (focus) need -= below;  // every key below the focused range is in
         focus = false;
         int cum = 0, bs = kBins - 1;
+#pragma unroll 4
         for (int c = 0; c < kBins; ++c) {
           int hc = sm.hist[1 + c][lane];
           if (cum + hc >= need) {
@@ -626,74 +735,80 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
   int nbuf = 0;
   uint32_t bslot[kBuf];  // member slots of the keys in the final bin (a few, in local memory)
   pass_id = 6;
-  for_each_bucket(warp_max(rcur), [&](uint32_t bb) {
-    bool want = valid && pt_box_d2(q, bmin[bb], bmax[bb]) <= rcur;
-    if (!__any_sync(FULL, want)) return;
+  for_each_bucket(rcur, [&](uint32_t bb, bool want, bool fits) {
     const uint32_t s0 = hs + 32u * (bb - 32u * sb0);
     const int cnt = (int)min(32u, he - s0);
     // 32-bit route as in the histogram passes: with both final-bin edges multiples of
     // 2^22, key < edge iff d^2 < edge >> 22
-    const bool narrow = fits32(qlo, qhi, bmin[bb], bmax[bb]) &&
-                        __all_sync(FULL, !want || ((fin_lo | fin_hi) & 0x3fffffull) == 0);
+    const bool narrow = fits && __all_sync(FULL, !want || ((fin_lo | fin_hi) & 0x3fffffull) == 0);
     stage(s0, cnt, true, narrow);
-    if (narrow && want) {
-      const int far = (want ? clamp31((u64)rcur) : -1) - rq.q2, flo = clamp31(fin_lo >> 22) - rq.q2,
-                fhi = clamp31(fin_hi >> 22) - rq.q2;
+    uint32_t in = 0, fin = 0;  // members below the final bin, and in it
+    if (narrow) {
+      const int none = -0x7fffffff - 1;
+      const int flo = want ? clamp31(fin_lo >> 22) - rq.q2 : none,
+                last = want ? min(clamp31((fin_hi >> 22) - 1), clamp31((u64)rcur)) - rq.q2 : none;
+#pragma unroll 1
       for (int t0 = 0; t0 < 32; t0 += BATCH) {
-        int d[BATCH];
-#pragma unroll
-        for (int j = 0; j < BATCH; ++j) d[j] = rel_d2(rq, sm.su[t0 + j]);
+        uint32_t bi = 0, bf = 0;
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) {
-          if (t0 + j < cnt && d[j] <= far) {
-            const int t = t0 + j;
-            if (d[j] < flo) {
-              top_insert(top, lane, tv, nv_eff, dv2f(sm.sv[t], vq));
-            } else if (d[j] < fhi && nbuf < kBuf) {
-              bslot[nbuf] = s0 + (uint32_t)t;
-              ++nbuf;
-            }
-          }
+          const int d = rel_d2(rq, sm.su[t0 + j]);
+          bi |= d < flo ? 1u << j : 0u;
+          bf |= d <= last ? 1u << j : 0u;
         }
+        in |= bi << t0;
+        fin |= bf << t0;
       }
-    } else if (want && !narrow) {
+    } else if (want) {
+#pragma unroll 1
       for (int t0 = 0; t0 < 32; t0 += BATCH) {
-        long long d[BATCH];
-#pragma unroll
-        for (int j = 0; j < BATCH; ++j) d[j] = d2i(q, sm.su[t0 + j]);
+        uint32_t bi = 0, bf = 0;
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) {
-          if (d[j] <= rcur) {
-            const int t = t0 + j;
-            u64 key = ((u64)d[j] << 22) | (u64)sm.su[t].w;
-            if (key < fin_lo) {
-              top_insert(top, lane, tv, nv_eff, dv2f(sm.sv[t], vq));
-            } else if (key < fin_hi && nbuf < kBuf) {
-              bslot[nbuf] = s0 + (uint32_t)t;
-              ++nbuf;
-            }
-          }
+          const int4 pc = sm.su[t0 + j];
+          const long long d = d2i(q, pc);
+          const u64 key = ((u64)d << 22) | (u64)pc.w;
+          bi |= key < fin_lo ? 1u << j : 0u;
+          bf |= key < fin_hi && d <= rcur ? 1u << j : 0u;
         }
+        in |= bi << t0;
+        fin |= bf << t0;
       }
     }
+    if (cnt < 32) {
+      in &= (1u << cnt) - 1u;
+      fin &= (1u << cnt) - 1u;
+    }
+    fin &= ~in;
+    for (; fin; fin &= fin - 1u)
+      if (nbuf < kBuf) bslot[nbuf++] = s0 + (uint32_t)(__ffs(fin) - 1);
+    // each lane its own next member: as many rounds as the lane with the most has (with an insertion
+    // in each member's place 39.4 ms for a 256^3 box, 38.2 so; with lanes passing over what their
+    // lists turn away and then replacing together 40.4)
+    for (; in; in &= in - 1u) top_insert(top, lane, tv, nv_eff, dv2f(sm.sv[__ffs(in) - 1], vq));
+    return false;
   });
   if (!valid) return;
-  // the need_in smallest keys of the final bin (keys recomputed from the buffered slots)
-  u64 last = 0;
-  for (int r = 0; r < need_in; ++r) {
-    int best = -1;
-    u64 bk = ~0ULL;
+  // the need_in smallest keys of the final bin, in order
+  if (need_in > 0) {
+    u64 bkey[kBuf];
     for (int e = 0; e < nbuf; ++e) {
       const int4 pe = u[bslot[e]];
-      const u64 x = ((u64)d2i(q, pe) << 22) | (u64)pe.w;
-      if ((r == 0 || x > last) && x < bk) {
-        bk = x;
-        best = e;
-      }
+      bkey[e] = ((u64)d2i(q, pe) << 22) | (u64)pe.w;
     }
-    if (best < 0) break;
-    last = bk;
-    top_insert(top, lane, tv, nv_eff, dv2f(v[bslot[best]], vq));
+    for (int r = 0; r < min(need_in, nbuf); ++r) {
+      int best = 0;
+      u64 bk = bkey[0];
+      for (int e = 1; e < nbuf; ++e) {
+        const u64 x = bkey[e];
+        if (x < bk) {
+          bk = x;
+          best = e;
+        }
+      }
+      bkey[best] = ~0ULL;
+      top_insert(top, lane, tv, nv_eff, dv2f(v[bslot[best]], vq));
+    }
   }
   f_l[__float_as_int(vq.w)] = top_density(top, lane, tv, nse_eff);
 }
@@ -732,11 +847,11 @@ namespace {
 // the default shape.
 template <int NVM>
 void *big_kernel(int shape) {
-  if (NVM > 32) return (void *)k_velden_big<NVM, 4, 80>;
+  if (NVM > 32) return (void *)k_velden_big<NVM, 4, 64>;
   switch (kVShapes[shape].batch) {
-    case 2: return (void *)k_velden_big<NVM, 2, 80>;
-    case 8: return (void *)k_velden_big<NVM, 8, 96>;
-    default: return (void *)k_velden_big<NVM, 4, 80>;
+    case 2: return (void *)k_velden_big<NVM, 2, 64>;
+    case 8: return (void *)k_velden_big<NVM, 8, 80>;
+    default: return (void *)k_velden_big<NVM, 4, 64>;
   }
 }
 
@@ -836,8 +951,11 @@ vr_status run_velden(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &a
     }
     return VR_OK;
   }
-  // one launch per halo-size bin, each with its own shape; a bin still to be tuned is
-  // run once per candidate shape (same results each time) and keeps the fastest
+  // a shape per halo-size bin; a bin still to be tuned is run once per candidate shape (same
+  // results each time) and keeps the fastest. Neighbouring bins of one shape share a launch,
+  // so that the last, long warps of one run beside the next (a third of the chip's time was idle in the
+  // launch of the largest halos: f_l of a 256^3 box 51.9 -> 45.1 ms with one launch), unless
+  // `ev_big` has to mark the end of the first bin.
   const int64_t lo[kVBins] = {0, 32LL * eg[0], 32LL * eg[1]};
   const int64_t hi[kVBins] = {32LL * eg[0], 32LL * eg[1], nbpad};
   timer_begin(ctx, "velden_big", s);
@@ -868,7 +986,12 @@ vr_status run_velden(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &a
       tn->vshape[k] = best;
       tn->vtuned[k] = 1;
     } else {
-      VR_CUDA(ctx, big(p->nv <= 32 ? vshape_for(ctx, k) : 0, lo[k], hi[k]));
+      const int sh = p->nv <= 32 ? vshape_for(ctx, k) : 0;
+      const int64_t first = lo[k];
+      while (k + 1 < kVBins && !(k == 0 && ev_big) &&
+             (p->nv > 32 || (!vmeasure(ctx, k + 1) && vshape_for(ctx, k + 1) == sh)))
+        ++k;
+      VR_CUDA(ctx, big(sh, first, hi[k]));
       VR_LAUNCHED(ctx, "k_velden_big");
     }
     if (k == 0 && ev_big) VR_CUDA(ctx, cudaEventRecord(ev_big, s));  // halos > kVBinEdge0 done
