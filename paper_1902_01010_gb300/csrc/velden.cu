@@ -23,7 +23,7 @@
 // wherever the two boxes involved (query bucket and candidate bucket or window) bound
 // every separation by kNarrow lattice units per axis, which makes them exact in 32 bits.
 //
-// What bounds the pass over a 256^3 box (36 ms): the issue slots (71 % taken at 5 warps a
+// What bounds the pass over a 256^3 box (34 ms): the issue slots (71 % taken at 5 warps a
 // scheduler), by phase the window's bound 7 %, the histogram levels 38 %, the collect pass 42 %
 // (most of it list insertions, whose lanes diverge), the keys of the final bin 13 %. Its code has
 // to stay small: with every loop over 32 members unrolled whole, warps in different phases put
@@ -613,16 +613,16 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       const int cnt = (int)min(32u, he - s0);
       // 32-bit route: the boxes are near enough and the bins of every lane are whole units of
       // d^2, so a key's bin depends on d^2 alone (klo is a multiple of 2^22): bin =
-      // (d^2 - (klo >> 22)) >> (sh - 22)
-      const bool narrow = fits && __all_sync(FULL, !want || (sh >= 22 && sh < 53 && (klo & 0x3fffffull) == 0));
+      // (d^2 - (klo >> 22)) >> (sh - 22), and its row one more (65 << (sh - 22) fits 31 bits)
+      const bool narrow = fits && __all_sync(FULL, !want || (sh >= 22 && sh < 47 && (klo & 0x3fffffull) == 0));
       stage(s0, cnt, false, narrow);
       if (narrow) {
         // without a branch per member: what lies below the bins or beyond the bound (all of it
         // for a lane that wants none) counts in a row of its own (f_l of a 256^3 box: 54.3 ms
         // with a compare and a branch for each, 51.8 so)
-        const int far = (want ? clamp31((u64)rlev) : -1) - rq.q2, off = rq.q2 - clamp31(klo >> 22);
-        const int shd = want ? sh - 22 : 0;
-        auto row_of = [&](int x) { return x > far ? kBins + 1 : max((x + off) >> shd, -1) + 1; };
+        const int far = (want ? clamp31((u64)rlev) : -1) - rq.q2, shd = want ? sh - 22 : 0;
+        const uint32_t off = (uint32_t)rq.q2 - (uint32_t)clamp31(klo >> 22) + (1u << shd);
+        auto row_of = [&](int x) { return x > far ? kBins + 1 : max((int)((uint32_t)x + off) >> shd, 0); };
         int d[BATCH];
 #pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
@@ -660,9 +660,9 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
           }
         }
       }
-      // Every 32 buckets: the bins counted so far bound the N_se-th key already, and nothing beyond
+      // Every 16 buckets: the bins counted so far bound the N_se-th key already, and nothing beyond
       // the bin that reaches it matters.
-      if (++visits & 31) return false;
+      if (++visits & 15) return false;
       if (rlev >= 0) {
         int cum = below + (int)sm.hist[0][lane];
         if (!focus) cum = 0;
@@ -782,6 +782,18 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     fin &= ~in;
     for (; fin; fin &= fin - 1u)
       if (nbuf < kBuf) bslot[nbuf++] = s0 + (uint32_t)(__ffs(fin) - 1);
+    // What the lists turn away already is passed over side by side first, where that is most of it:
+    // of N_se members a list takes about N_v (1 + ln(N_se / N_v)). f_l of a 256^3 box (256 and 32)
+    // 35.5 -> 34.4 ms; with 64 and 16, where the lists take 60 %, 24.1 -> 24.4, so not there.
+    if (nse_eff >= 6 * nv_eff && __reduce_max_sync(FULL, (unsigned)__popc(in)) > 10u) {
+      uint32_t drop = 0;
+#pragma unroll 1
+      for (uint32_t some = __reduce_or_sync(FULL, in); some; some &= some - 1u) {
+        const int k = __ffs(some) - 1;
+        drop |= dv2f(sm.sv[k], vq) < tv.m ? 0u : 1u << k;
+      }
+      if (tv.c >= nv_eff) in &= ~drop;
+    }
     // each lane its own next member: as many rounds as the lane with the most has (with an insertion
     // in each member's place 39.4 ms for a 256^3 box, 38.2 so; with lanes passing over what their
     // lists turn away and then replacing together 40.4)
