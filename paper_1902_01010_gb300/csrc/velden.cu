@@ -9,11 +9,12 @@
 //    its N_se-th neighbour distance by the N_se-th smallest distance among the 4 N_se
 //    members around the bucket in Morton order (to within one of 64 histogram bins);
 //    every later pass visits only the buckets whose boxes come within the largest
-//    per-lane bound of the warp's own box (super-bucket boxes prune first);
+//    per-lane bounds of the boxes of the warp's two parts (super-bucket boxes prune first),
+//    and within some lane's bound of that lane;
 //  - each visited bucket is staged once in shared memory and read back by every lane
 //    with broadcast 16-byte loads; every lane keeps its own 64-bin histogram of the exact
 //    key (d^2 << 22 | local index). Histogram passes narrow the key range until the bin
-//    holding the N_se-th key has at most 16 keys; a last pass feeds every key below that
+//    holding the N_se-th key has at most 32 keys; a last pass feeds every key below that
 //    bin, plus the right number from the bin, into a per-lane list of the N_v smallest
 //    |dv|^2 (shared memory);
 //  - h^2 is the largest kept |dv|^2, and the kernel sum runs over the kept list only
@@ -23,7 +24,7 @@
 // wherever the two boxes involved (query bucket and candidate bucket or window) bound
 // every separation by kNarrow lattice units per axis, which makes them exact in 32 bits.
 //
-// What bounds the pass over a 256^3 box (34 ms): the issue slots (71 % taken at 5 warps a
+// What bounds the pass over a 256^3 box (34 ms): the issue slots (76 % taken at 7 warps a
 // scheduler), by phase the window's bound 7 %, the histogram levels 38 %, the collect pass 42 %
 // (most of it list insertions, whose lanes diverge), the keys of the final bin 13 %. Its code has
 // to stay small: with every loop over 32 members unrolled whole, warps in different phases put
@@ -486,14 +487,14 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     r2 = (((long long)bs + 1) << sh0) - 1;  // every distance in bins <= bs is <= r2
     if (r2 > wmax) r2 = wmax;
   }
-  if (r2 >= (1LL << 41)) {
-    raise_error(st, VR_ERR_UNSUPPORTED, 1);
+  if (__any_sync(FULL, r2 >= (1LL << 41))) {  // all lanes leave, so that none waits for one that left
+    if (r2 >= (1LL << 41)) raise_error(st, VR_ERR_UNSUPPORTED, 1);
     return;
   }
   // Two parts of the query bucket: where the curve jumps, its particles lie in two clumps, and
   // one box would reach everything between them (in a halo of 564 k members one bucket
-  // tested 27,000 others one by one for 437 to visit: 25 M cycles, 13 ms, as long as the launch's
-  // other warps together; with two parts 6 M).
+  // tested 27,000 others one by one for 437 to visit: 25 M cycles, 13 ms, a third of the whole
+  // launch; the longest warp of any is 9 M cycles with two parts).
   // Boxes of the particles up to each lane and from each lane on; the cut is where the two
   // volumes are least, each extent with an eighth of the largest one added.
   int cut = 31;
