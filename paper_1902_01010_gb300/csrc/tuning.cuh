@@ -23,7 +23,7 @@ constexpr int kLWarps[kNLShapes] = {4, 2, 8};
 
 struct Tuning {
   int on = 0;                       // measure each untuned bin at its next launch
-  int vshape[kVBins] = {0, 0, 0};   // chosen f_l shape per bin (0 = default)
+  int vshape[kVBins] = {0, 0, 0};   // chosen f_l shape per tuned bin
   int vtuned[kVBins] = {0, 0, 0};
   float vms[kVBins][kNVShapes] = {};
   int lshape = 0, ltuned = 0;       // chosen linker shape
@@ -31,12 +31,17 @@ struct Tuning {
   int force_v = -1, force_l = -1;   // every launch uses this shape (tests), -1 = off
 };
 
-// Shape index for f_l bin k / the linker under the context's tuning state.
-inline int vshape_for(const vr_ctx *ctx, int k) {
+// Shape index for f_l bin k / the linker under the context's tuning state. Untuned f_l
+// launches of many buckets take 2 warps per block, whose places are free again sooner (256^3 box,
+// 150,000 buckets: 33.3 ms with 4 warps, 32.6 with 2; a catalogue of 180,000: 23.2 and 22.7); of
+// few buckets 4, of which more start at once (1M particles, 8,900 buckets: 3.39 and 3.44).
+constexpr int64_t kVManyBuckets = 32768;
+constexpr int kVShapeMany = 2;
+inline int vshape_for(const vr_ctx *ctx, int k, int64_t buckets = 0) {
   const Tuning *t = ctx ? ctx->tune : nullptr;
-  if (!t) return 0;
-  if (t->force_v >= 0) return t->force_v;
-  return t->vtuned[k] ? t->vshape[k] : 0;
+  if (t && t->force_v >= 0) return t->force_v;
+  if (t && t->vtuned[k]) return t->vshape[k];
+  return buckets >= kVManyBuckets ? kVShapeMany : 0;
 }
 inline int lshape_for(const vr_ctx *ctx) {
   const Tuning *t = ctx ? ctx->tune : nullptr;

@@ -24,7 +24,7 @@
 // wherever the two boxes involved (query bucket and candidate bucket or window) bound
 // every separation by kNarrow lattice units per axis, which makes them exact in 32 bits.
 //
-// What bounds the pass over a 256^3 box (34 ms): the issue slots (76 % taken at 7 warps a
+// What bounds the pass over a 256^3 box (33 ms): the issue slots (76 % taken at 7 warps a
 // scheduler), by phase the window's bound 7 %, the histogram levels 38 %, the collect pass 42 %
 // (most of it list insertions, whose lanes diverge), the keys of the final bin 13 %. Its code has
 // to stay small: with every loop over 32 members unrolled whole, warps in different phases put
@@ -46,6 +46,11 @@ constexpr int kNVMax = 64;
 constexpr int kBinBits = 6;      // histogram levels resolve kBinBits bits of the key
 constexpr int kBins = 1 << kBinBits;
 constexpr int kBuf = 32;
+// Lanes that want a bucket, up to which the collect pass takes it a lane per member and query by
+// query (about 22 instructions a query) instead of a lane per query (about 300 for the 32 members):
+// f_l of a 256^3 box 34.5 -> 33.3 ms, of a catalogue with N_se 64 24.2 -> 23.2. In the levels, where
+// the counts then need shared-memory atomics, the same gained nothing (34.4 to 34.7).
+constexpr int kFewLanes = 12;
 constexpr int kWarps = 4;        // warps per block
 
 // Optional instrumentation (compile with -DVR_VELDEN_STATS): warp-level counts of the
@@ -744,21 +749,54 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     const bool narrow = fits && __all_sync(FULL, !want || ((fin_lo | fin_hi) & 0x3fffffull) == 0);
     stage(s0, cnt, true, narrow);
     uint32_t in = 0, fin = 0;  // members below the final bin, and in it
+    const unsigned who = __ballot_sync(FULL, want);
+    const bool few = __popc(who) <= kFewLanes;
     if (narrow) {
       const int none = -0x7fffffff - 1;
       const int flo = want ? clamp31(fin_lo >> 22) - rq.q2 : none,
                 last = want ? min(clamp31((fin_hi >> 22) - 1), clamp31((u64)rcur)) - rq.q2 : none;
+      if (few) {  // a lane per member, query by query
+        const int4 c = sm.su[lane];
 #pragma unroll 1
-      for (int t0 = 0; t0 < 32; t0 += BATCH) {
-        uint32_t bi = 0, bf = 0;
-#pragma unroll
-        for (int j = 0; j < BATCH; ++j) {
-          const int d = rel_d2(rq, sm.su[t0 + j]);
-          bi |= d < flo ? 1u << j : 0u;
-          bf |= d <= last ? 1u << j : 0u;
+        for (unsigned w = who; w; w &= w - 1u) {
+          const int l = __ffs(w) - 1;
+          Rel o;
+          o.ax = __shfl_sync(FULL, rq.ax, l);
+          o.ay = __shfl_sync(FULL, rq.ay, l);
+          o.az = __shfl_sync(FULL, rq.az, l);
+          const int d = rel_d2(o, c), ofl = __shfl_sync(FULL, flo, l), ola = __shfl_sync(FULL, last, l);
+          const unsigned bi = __ballot_sync(FULL, d < ofl), bf = __ballot_sync(FULL, d <= ola);
+          in = lane == l ? bi : in;
+          fin = lane == l ? bf : fin;
         }
-        in |= bi << t0;
-        fin |= bf << t0;
+      } else {
+#pragma unroll 1
+        for (int t0 = 0; t0 < 32; t0 += BATCH) {
+          uint32_t bi = 0, bf = 0;
+#pragma unroll
+          for (int j = 0; j < BATCH; ++j) {
+            const int d = rel_d2(rq, sm.su[t0 + j]);
+            bi |= d < flo ? 1u << j : 0u;
+            bf |= d <= last ? 1u << j : 0u;
+          }
+          in |= bi << t0;
+          fin |= bf << t0;
+        }
+      }
+    } else if (few) {
+      const int4 c = sm.su[lane];
+#pragma unroll 1
+      for (unsigned w = who; w; w &= w - 1u) {
+        const int l = __ffs(w) - 1;
+        const int4 o = make_int4(__shfl_sync(FULL, q.x, l), __shfl_sync(FULL, q.y, l), __shfl_sync(FULL, q.z, l), 0);
+        const long long d = d2i(o, c);
+        const u64 key = ((u64)d << 22) | (u64)c.w, olo = __shfl_sync(FULL, fin_lo, l);
+        const unsigned bi = __ballot_sync(FULL, key < olo);
+        const u64 ohi = __shfl_sync(FULL, fin_hi, l);
+        const long long orc = __shfl_sync(FULL, rcur, l);
+        const unsigned bf = __ballot_sync(FULL, key < ohi && d <= orc);
+        in = lane == l ? bi : in;
+        fin = lane == l ? bf : fin;
       }
     } else if (want) {
 #pragma unroll 1
@@ -999,10 +1037,10 @@ vr_status run_velden(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &a
       tn->vshape[k] = best;
       tn->vtuned[k] = 1;
     } else {
-      const int sh = p->nv <= 32 ? vshape_for(ctx, k) : 0;
+      const int sh = p->nv <= 32 ? vshape_for(ctx, k, nbpad) : 0;
       const int64_t first = lo[k];
       while (k + 1 < kVBins && !(k == 0 && ev_big) &&
-             (p->nv > 32 || (!vmeasure(ctx, k + 1) && vshape_for(ctx, k + 1) == sh)))
+             (p->nv > 32 || (!vmeasure(ctx, k + 1) && vshape_for(ctx, k + 1, nbpad) == sh)))
         ++k;
       VR_CUDA(ctx, big(sh, first, hi[k]));
       VR_LAUNCHED(ctx, "k_velden_big");
