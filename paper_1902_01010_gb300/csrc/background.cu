@@ -1033,6 +1033,7 @@ __global__ void __launch_bounds__(NT) __cluster_dims__(kTeam, 1, 1) k_cells_clus
     }
     __syncthreads();
   }
+  cl.sync();  // the others may still read the first block's s_child, which it writes below
   WarpTree *wt = reinterpret_cast<WarpTree *>(tree_smem);
   for (int k = part; k < nlist; k += kTeam) {
     const int id = s_list[k];

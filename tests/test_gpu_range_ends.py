@@ -1,0 +1,65 @@
+"""Calls at the ends of what the library accepts and at the hand-overs inside its kernels,
+on the GPU vs the oracle or a plain numpy form of the same step. No case faults the GPU:
+what is out of range is refused by the host or by a kernel's own check.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+L = 1 << 21
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1902_01010_gb300 import Context
+
+    return Context(0)
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# ------------------------------------------------------------ trees built by a cluster
+def test_cluster_trees_hand_over_to_their_blocks(ctx):
+    """Halos whose nodes a cluster splits together before each block takes subtrees of its
+    own: equal coordinates make the halves uneven, so the cluster's last split comes at
+    another node in each halo and the blocks start on subtrees of different sizes. Every
+    build gives the same cells and the same bits of R; the cells are the oracle's."""
+    from paper_1902_01010_gb300 import Params
+
+    rng = np.random.default_rng(2)
+    sizes, steps = [65536, 70001, 90000, 131072], [1, 9000, 2500, 20000]
+    pos, vel, lab, at = [], [], [], 0
+    for k, (n, step) in enumerate(zip(sizes, steps)):
+        p = np.round(rng.normal(0, 40000 / step, size=(n, 3))).astype(np.int64) * step
+        pos.append((p + 400000 * k) % L)
+        vel.append(rng.normal(0, 80, size=(n, 3)))
+        lab.append(np.full(n, at))
+        at += n
+    pos = np.concatenate(pos).astype(np.int32)
+    vel = np.concatenate(vel).astype(np.float32)
+    lab = np.concatenate(lab).astype(np.int32)
+    fl = np.exp(rng.normal(-12, 1, at)).astype(np.float32)
+    d = [_dev(pos), _dev(vel), _dev(fl), _dev(lab)]
+    first = None
+    for _ in range(20):
+        R, _, hs = ctx.outlier_ratio(*d, Params.default())
+        ctx.sync()
+        got = R.cpu().numpy(), hs.cpu().numpy()[:, 11]
+        if first is None:
+            first = got
+        assert np.array_equal(got[0], first[0], equal_nan=True) and np.array_equal(got[1], first[1])
+    o = 0
+    for k, n in enumerate(sizes):
+        m = np.arange(o, o + n)
+        ref, leaf, _ = oracle.background_halo(oracle.unwrap(pos, m), vel, m, fl[m].astype(np.float64))
+        assert first[1][k] == len(np.unique(leaf))
+        fin = np.isfinite(ref)
+        assert np.array_equal(np.isfinite(first[0][m]), fin)
+        assert (np.abs(first[0][m][fin] - ref[fin]) <= 1e-4 * np.maximum(1.0, np.abs(ref[fin]))).all()
+        o += n
