@@ -81,8 +81,8 @@ __global__ void k_member_flags(const int32_t *__restrict__ label, const uint32_t
     mflag[n] = 0;
     return;
   }
-  uint32_t c = cnt[label[i]];
-  mflag[i] = (c >= (uint32_t)nmin) ? 1u : 0u;
+  const int32_t l = label[i];  // outside [0, n): k_count's error ends the call after this kernel
+  mflag[i] = l >= 0 && l < n && cnt[l] >= (uint32_t)nmin ? 1u : 0u;
 }
 
 // Compacts halo members in index order with key = halo id.

@@ -63,3 +63,34 @@ def test_cluster_trees_hand_over_to_their_blocks(ctx):
         assert np.array_equal(np.isfinite(first[0][m]), fin)
         assert (np.abs(first[0][m][fin] - ref[fin]) <= 1e-4 * np.maximum(1.0, np.abs(ref[fin]))).all()
         o += n
+
+
+# ------------------------------------------------------------------ labels out of range
+@pytest.mark.parametrize("bad", [-1, -(1 << 31), 5000, (1 << 31) - 1])
+@pytest.mark.parametrize("call", ["velden", "fof6d_field", "find_substructure"])
+def test_label_out_of_range_is_refused(ctx, call, bad):
+    """One label outside [0, n) among 5,000: VR_ERR_INVALID_ARG, and the next call on the
+    context works."""
+    from paper_1902_01010_gb300 import VrError
+
+    rng = np.random.default_rng(3)
+    n = 5000
+    pos = _dev(rng.integers(0, 40000, size=(n, 3)).astype(np.int32))
+    vel = _dev(rng.normal(0, 50, (n, 3)).astype(np.float32))
+    good = np.zeros(n, np.int32)
+    want = ctx.velden(pos, vel, _dev(good))
+    ctx.sync()
+    lab = good.copy()
+    lab[3777] = bad
+    with pytest.raises(VrError) as e:
+        if call == "velden":
+            ctx.velden(pos, vel, _dev(lab))
+        elif call == "fof6d_field":
+            ctx.fof6d_field(pos, vel, _dev(lab), 1000.0)
+        else:
+            ctx.find_substructure(pos, vel, _dev(lab), 1000.0, 1.0)
+        ctx.sync()
+    assert e.value.code == 1 and "label" in str(e.value)
+    got = ctx.velden(pos, vel, _dev(good))
+    ctx.sync()
+    assert torch.equal(got, want)
