@@ -7,7 +7,9 @@
 //     particle without any distance test;
 //  2. link cells of 2 sub-cells per axis (side 2S >= linking length; the last link cell
 //     of each axis takes the 3 or 4 leftover sub-cells, so no link cell is thinner than
-//     the linking length across the periodic edge): every linked pair lies in the same or
+//     the linking length across the periodic edge; of 4 sub-cells for link_d2 <= 3, whose
+//     S = 1 would give more link cells than the sort key has bits for): every linked pair
+//     lies in the same or
 //     an adjacent link cell. Particles are ordered by (Morton code of the link cell,
 //     position of the sub-cell inside it) with the library's radix sort, which makes
 //     every sub-cell, link cell and coarse cell (2^q link cells per axis) one contiguous
@@ -50,7 +52,8 @@ constexpr uint32_t kEmpty = 0xffffffffu;
 struct FofGeom {
   int S;        // sub-cell side (lattice units)
   int G;        // sub-cells per axis (last one partial)
-  int GL;       // link cells per axis: 2 sub-cells each, the last one 3 or 4
+  int lw;       // a link cell is 2^lw sub-cells wide (the last one of an axis up to 4)
+  int GL;       // link cells per axis
   int bl;       // bits per axis of link-cell coordinates
   int q;        // coarse cell = 2^q link cells per axis
   int64_t ncoarse;
@@ -84,7 +87,10 @@ FofGeom fof_geom(int64_t link_d2, int64_t n) {
   FofGeom g;
   g.S = (int)isqrt64((link_d2 - 1) / 3) + 1;  // 3 (S-1)^2 <= link_d2 - 1 < link_d2
   g.G = (int)((kLattice + g.S - 1) / g.S);
-  g.GL = (g.G - 1) / 2;
+  // the sort key holds 6 + 3 bl bits: 19 bits per axis at most. With S = 1 (link_d2 <= 3) link
+  // cells of 2 would need 20, so they take 4, of which the 2^21 sub-cells leave no remainder
+  g.lw = g.S == 1 ? 2 : 1;
+  g.GL = g.S == 1 ? g.G / 4 : (g.G - 1) / 2;
   g.bl = 0;
   while ((1 << g.bl) < g.GL) ++g.bl;
   if (g.bl == 0) g.bl = 1;
@@ -126,9 +132,9 @@ FofBufs fof_carve(Arena &ar, int64_t n, int64_t ncoarse, int om) {
   return b;
 }
 
-// Sub-cell c of an axis lies in link cell min(c / 2, GL - 1) at position c - 2 * that.
-__device__ __forceinline__ uint32_t link_of(uint32_t c, int GL) {
-  uint32_t l = c >> 1;
+// Sub-cell c of an axis lies in link cell min(c >> lw, GL - 1) at position c - (that << lw).
+__device__ __forceinline__ uint32_t link_of(uint32_t c, int lw, int GL) {
+  uint32_t l = c >> lw;
   return l < (uint32_t)GL ? l : (uint32_t)GL - 1u;
 }
 
@@ -149,7 +155,7 @@ __device__ __forceinline__ uint32_t compact3(u64 x);
 
 // Sort key: Morton code of the link cell << 6 | 2-bit sub-cell position per axis. Link
 // cells (key >> 6) and coarse cells are its prefixes.
-__global__ void k_fof_keys(const int32_t *__restrict__ pos, int64_t n, int S, int GL,
+__global__ void k_fof_keys(const int32_t *__restrict__ pos, int64_t n, int S, int lw, int GL,
                            u64 *__restrict__ keys, uint32_t *__restrict__ vals) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -158,9 +164,9 @@ __global__ void k_fof_keys(const int32_t *__restrict__ pos, int64_t n, int S, in
   uint32_t x = ((uint32_t)pos[3 * i] & m) / (uint32_t)S,
            y = ((uint32_t)pos[3 * i + 1] & m) / (uint32_t)S,
            z = ((uint32_t)pos[3 * i + 2] & m) / (uint32_t)S;
-  uint32_t lx = link_of(x, GL), ly = link_of(y, GL), lz = link_of(z, GL);
-  keys[i] = (morton3(lx, ly, lz) << 6) | ((u64)(x - 2 * lx) << 4) | ((u64)(y - 2 * ly) << 2) |
-            (u64)(z - 2 * lz);
+  uint32_t lx = link_of(x, lw, GL), ly = link_of(y, lw, GL), lz = link_of(z, lw, GL);
+  keys[i] = (morton3(lx, ly, lz) << 6) | ((u64)(x - (lx << lw)) << 4) | ((u64)(y - (ly << lw)) << 2) |
+            (u64)(z - (lz << lw));
   vals[i] = (uint32_t)i;
 }
 
@@ -283,15 +289,15 @@ struct FofCells {
   const uint32_t *sid;
   const uint2 *ctab;
   const unsigned long long *occ;
-  int om, S, GL, qshift;
+  int om, S, lw, GL, qshift;
   long long T;
 };
 
-// Extent of sub-cell coordinates 2 l + (2-bit position of the sort key) per axis.
-__device__ __forceinline__ void sub_box(u64 key, const int *l, int S, int *lo, int *hi) {
-  cell_span(2 * l[0] + (int)((key >> 4) & 3u), S, lo[0], hi[0]);
-  cell_span(2 * l[1] + (int)((key >> 2) & 3u), S, lo[1], hi[1]);
-  cell_span(2 * l[2] + (int)(key & 3u), S, lo[2], hi[2]);
+// Extent of sub-cell coordinates (l << lw) + (2-bit position of the sort key) per axis.
+__device__ __forceinline__ void sub_box(u64 key, const int *l, int lw, int S, int *lo, int *hi) {
+  cell_span((l[0] << lw) + (int)((key >> 4) & 3u), S, lo[0], hi[0]);
+  cell_span((l[1] << lw) + (int)((key >> 2) & 3u), S, lo[1], hi[1]);
+  cell_span((l[2] << lw) + (int)(key & 3u), S, lo[2], hi[2]);
 }
 
 // Squared distance from x (inside A's box) to box B in A's frame.
@@ -308,8 +314,8 @@ __device__ __forceinline__ void pair_boxes(const FofCells &f, uint32_t a0, const
                                            const int *lb, int *bl, int *bh, long long &mind,
                                            long long &maxd) {
   int alo[3], ahi[3], lo[3], hi[3];
-  sub_box(f.keyS[a0], la, f.S, alo, ahi);
-  sub_box(f.keyS[b0], lb, f.S, lo, hi);
+  sub_box(f.keyS[a0], la, f.lw, f.S, alo, ahi);
+  sub_box(f.keyS[b0], lb, f.lw, f.S, lo, hi);
   mind = maxd = 0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -724,7 +730,7 @@ extern "C" vr_status vr_fof3d(vr_ctx *ctx, const int32_t *pos, int64_t n, int64_
   vr_status st = check_ws(ctx, ar, ws_bytes);
   if (st != VR_OK) return st;
   const int T = 256;
-  k_fof_keys<<<grid_for(n, T), T, 0, s>>>(pos, n, g.S, g.GL, B.k0, B.v0);
+  k_fof_keys<<<grid_for(n, T), T, 0, s>>>(pos, n, g.S, g.lw, g.GL, B.k0, B.v0);
   VR_LAUNCHED(ctx, "k_fof_keys");
   int which = 0;
   VR_CUDA(ctx, radix_sort_pairs<u64>(B.k0, B.v0, B.k1, B.v1, n, 0, 6 + 3 * g.bl, B.scratch, s,
@@ -751,7 +757,7 @@ extern "C" vr_status vr_fof3d(vr_ctx *ctx, const int32_t *pos, int64_t n, int64_
   uint32_t *nheavy = reinterpret_cast<uint32_t *>(B.scratch);
   uint2 *heavy = reinterpret_cast<uint2 *>(spare);
   VR_CUDA(ctx, cudaMemsetAsync(nheavy, 0, 2 * sizeof(uint32_t), s));
-  FofCells f{B.posS, keyS, B.sc_start, lcfirst, sid, B.ctab, B.occ, g.om, g.S, g.GL, qshift, (long long)link_d2};
+  FofCells f{B.posS, keyS, B.sc_start, lcfirst, sid, B.ctab, B.occ, g.om, g.S, g.lw, g.GL, qshift, (long long)link_d2};
   // link cells a warp takes at a time (n bounds their number): 32, or 64 warps per SM. Each
   // warp takes two such runs; more blocks than fit at once let the dense regions, which lie
   // together in sort order, spread over the SMs (k_fof_neigh at 512^3 with the resident

@@ -94,3 +94,25 @@ def test_label_out_of_range_is_refused(ctx, call, bad):
     got = ctx.velden(pos, vel, _dev(good))
     ctx.sync()
     assert torch.equal(got, want)
+
+
+# ------------------------------------------------- 3D FOF with the shortest linking lengths
+@pytest.mark.parametrize("T", [1, 2, 3, 4])
+@pytest.mark.parametrize("n", [0, 3000, 40000])
+def test_fof_shortest_linking_lengths(ctx, T, n):
+    """Sub-cells of one lattice point. Points that differ by half the box along any axes share
+    all but the top bit of each coordinate; around them clumps of lattice neighbours, across
+    the periodic edge too, and cells of more members than one warp tests at once."""
+    rng = np.random.default_rng(10 * T + n)
+    h = 1 << 20
+    corners = np.stack(np.meshgrid(*[[0, h]] * 3, indexing="ij"), -1).reshape(-1, 3) + 5
+    pos = [corners, corners, corners + [1, 0, 0], corners + [0, 1, 1], corners - 6]
+    if n:
+        ctr = np.concatenate([rng.integers(0, L, size=(20, 3)), [[0, 0, 0], [h, h, h], [L - 1, 3, h - 1]]])
+        pos.append(ctr[rng.integers(0, len(ctr), n)] + rng.integers(-6, 7, size=(n, 3)))
+        pos.append(rng.integers(0, L, size=(n // 3, 3)))
+    pos = (np.concatenate(pos) % L).astype(np.int32)
+    pos = pos[rng.permutation(len(pos))]
+    lab = ctx.fof3d(_dev(pos), T)
+    ctx.sync()
+    assert np.array_equal(lab.cpu().numpy(), oracle.fof3d(pos, T))
