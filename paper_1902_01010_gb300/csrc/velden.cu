@@ -46,6 +46,9 @@ constexpr int kNVMax = 64;
 constexpr int kBinBits = 6;      // histogram levels resolve kBinBits bits of the key
 constexpr int kBins = 1 << kBinBits;
 constexpr int kBuf = 32;
+// A bin's 16-bit count is held at kFull: above N_se + kBuf (1,024 + 32) its value no longer
+// matters, and 16 buckets add at most 512 before it is looked at again.
+constexpr int kFull = 32768;
 // Lanes that want a bucket, up to which the collect pass takes it a lane per member and query by
 // query (about 22 instructions a query) instead of a lane per query (about 300 for the 32 members):
 // f_l of a 256^3 box 34.5 -> 33.3 ms, of a catalogue with N_se 64 24.2 -> 23.2. In the levels, where
@@ -609,7 +612,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
   bool focus = true;    // this lane's current level is the focused first level
   for (int level = 0; level < 16; ++level) {
     pass_id = level < 5 ? 1 + level : 5;
-    int below = 0, seen = 0, visits = 0;
+    int below = 0, visits = 0;
     long long rlev = settled ? -1 : rcur;  // bound on d^2 of the keys that this level has to count
     if (!settled)
 #pragma unroll 4
@@ -638,14 +641,6 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
           for (int j = 0; j < BATCH; ++j) sm.hist[row_of(d[j])][lane]++;
         }
         sm.hist[row_of(d[BATCH - 1])][lane] -= 32 - cnt;  // the repeated last one
-        seen += 32;
-        if (seen > 0xffff - 32) {  // before the 16-bit count of row 0 could wrap
-          seen = 0;
-          if (!settled) {
-            below += sm.hist[0][lane];
-            sm.hist[0][lane] = 0;
-          }
-        }
       } else if (want) {
 #pragma unroll 1
         for (int t0 = 0; t0 < 32; t0 += BATCH) {
@@ -667,7 +662,9 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
         }
       }
       // Every 16 buckets: the bins counted so far bound the N_se-th key already, and nothing beyond
-      // the bin that reaches it matters.
+      // the bin that reaches it matters. The count of that bin is held at kFull, since the buckets
+      // to come may hold more of its keys than 16 bits count (a halo has up to 2^22 members, and
+      // coincident ones all fall in one bin); the rows before it hold fewer than N_se in all.
       if (++visits & 15) return false;
       if (rlev >= 0) {
         int cum = below + (int)sm.hist[0][lane];
@@ -677,8 +674,10 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
         } else {
 #pragma unroll 4
           for (int c = 0; c < kBins; ++c) {
-            cum += sm.hist[1 + c][lane];
+            const int hc = sm.hist[1 + c][lane];
+            cum += hc;
             if (cum >= need) {
+              if (hc > kFull) sm.hist[1 + c][lane] = (uint16_t)kFull;
               const long long top_d = (long long)((klo + ((u64)(c + 1) << sh) - 1) >> 22);
               rlev = top_d < rlev ? top_d : rlev;
               break;

@@ -116,3 +116,32 @@ def test_fof_shortest_linking_lengths(ctx, T, n):
     lab = ctx.fof3d(_dev(pos), T)
     ctx.sync()
     assert np.array_equal(lab.cpu().numpy(), oracle.fof3d(pos, T))
+
+
+# ---------------------------------------- f_l: more members in one bin than 16 bits count
+@pytest.mark.parametrize("n,near,gap,spread", [
+    (65536, 0, 0, 0), (70000, 0, 0, 0), (131072, 0, 0, 0),          # all at one point
+    (65600, 100, 5000, 0), (65600, 100, 40000, 0),                  # all at one distance
+    (65700, 40, 5000, 2), (131200, 100, 40000, 2), (66000, 255, 20000, 30)])
+def test_fl_bins_of_more_than_16_bits(ctx, n, near, gap, spread):
+    """`n` members in a clump and `near` others at a distance of `gap`, for which the whole clump
+    lies in one bin of a level; N_se = 256 of them decided by the particle index where the
+    separations are equal."""
+    from paper_1902_01010_gb300 import Params
+
+    rng = np.random.default_rng(n + gap)
+    p = np.concatenate([[gap, 0, 0] + np.round(rng.uniform(-spread, spread, (n, 3))),
+                        np.round(rng.uniform(-20, 20, (near, 3)))]).astype(np.int64)
+    p = p[rng.permutation(len(p))]
+    pos = ((p + 700000) % L).astype(np.int32)
+    vel = rng.normal(0, 80, size=pos.shape).astype(np.float32)
+    lab = np.zeros(len(pos), np.int32)
+    got = ctx.velden(_dev(pos), _dev(vel), _dev(lab), Params.default())
+    ctx.sync()
+    got = got.cpu().numpy()
+    m = np.arange(len(pos))
+    up = oracle.unwrap(pos, m)
+    few = np.flatnonzero(p[:, 0] < gap - spread)
+    for k in np.r_[rng.integers(0, len(pos), 12), few[:24]].astype(int):
+        ref = oracle.velden_one(up, vel, m, int(k))
+        assert abs(got[k] - ref) <= 1e-4 * ref, k
