@@ -623,8 +623,12 @@ vr_status run_fit(vr_ctx *ctx, const HaloSeg &g, const Background &bg, const vr_
   if (hoff_host) szlo = 0, szhi = 0xffffffffu;
   k_gather_r<<<grid_for(g.NHP, 256), 256, 0, s>>>(g.v, R, g.NHP, g.hid, g.hoff, szlo, szhi, Rs);
   VR_LAUNCHED(ctx, "k_gather_r");
-  const size_t lm_smem = (size_t)kLmWarps * 2 * p->fit_nbins_max * sizeof(double);
-  VR_CUDA(ctx, cudaFuncSetAttribute(k_fit_lm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm_smem));
+  // the attribute belongs to the function, not to this call: it is the same for every context, so
+  // that another host thread's call cannot lower it between here and the launch
+  constexpr size_t kLmRow = (size_t)kLmWarps * 2 * sizeof(double);
+  VR_CUDA(ctx, cudaFuncSetAttribute(k_fit_lm, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kLmRow * kMaxFitBins)));
+  const size_t lm_smem = kLmRow * p->fit_nbins_max;
   // halos [a, z) of the size order; the large ones are its first, at most NHP / kFitBig
   auto fit = [&](int64_t a, int64_t z) -> vr_status {
     const int64_t nbig = g.NHP / kFitBig, zb = nbig < z ? nbig : z;

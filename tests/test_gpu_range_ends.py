@@ -145,3 +145,51 @@ def test_fl_bins_of_more_than_16_bits(ctx, n, near, gap, spread):
     for k in np.r_[rng.integers(0, len(pos), 12), few[:24]].astype(int):
         ref = oracle.velden_one(up, vel, m, int(k))
         assert abs(got[k] - ref) <= 1e-4 * ref, k
+
+
+# ------------------------------------------------------- contexts on several host threads
+def test_contexts_on_host_threads_with_different_bin_counts():
+    """One context per host thread is a documented use: calls with few and with many fit bins
+    at the same time all succeed and give what each gives alone."""
+    import ctypes
+    import threading
+
+    from paper_1902_01010_gb300 import Context, Params, lib
+    from paper_1902_01010_gb300.vr import HALO_COLS, _ptr
+
+    rng = np.random.default_rng(9)
+    n = 300
+    pos = _dev((np.round(rng.normal(0, 30000, (n, 3))).astype(np.int64) % L).astype(np.int32))
+    vel = _dev(rng.normal(0, 80, (n, 3)).astype(np.float32))
+    fl = _dev(np.exp(rng.normal(-12, 1, n)).astype(np.float32))
+    lab = torch.zeros(n, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    bins = [1024, 1024] + 6 * [200]
+    alone = {b: Context(0).outlier_ratio(pos, vel, fl, lab, Params.default(fit_nbins_max=b))[1].cpu()
+             for b in set(bins)}
+    errors, call = [], lib().vr_outlier_ratio
+    start = threading.Barrier(len(bins))
+
+    def work(b):
+        try:
+            c, s, P, nh = Context(0), torch.cuda.Stream(), Params.default(fit_nbins_max=b), ctypes.c_int64()
+            with torch.cuda.stream(s):
+                ws = c.workspace(n, P)
+                R, ell = (torch.empty(n, dtype=torch.float32, device="cuda") for _ in range(2))
+                hs = torch.empty((n // P.nmin + 1, HALO_COLS), dtype=torch.float64, device="cuda")
+            args = (c.h, _ptr(pos), _ptr(vel), _ptr(fl), n, _ptr(lab), ctypes.byref(P), _ptr(R), _ptr(ell),
+                    _ptr(hs), ctypes.byref(nh), _ptr(ws), ws.numel(), ctypes.c_void_p(s.cuda_stream))
+            start.wait()
+            for _ in range(1000):
+                c.check(call(*args))
+            s.synchronize()
+            assert torch.equal(ell.cpu(), alone[b])
+        except Exception as e:  # noqa: BLE001
+            errors.append(f"{b} bins: {e}")
+
+    threads = [threading.Thread(target=work, args=(b,)) for b in bins]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
