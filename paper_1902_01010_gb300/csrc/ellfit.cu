@@ -230,10 +230,12 @@ __device__ unsigned long long block_prev_rank(int n, int k, unsigned long long a
 // k-th smallest |x - med| (exact FP64 values), and with `even` the one before it: median of
 // the two. FP32 distances d_f = |x - med_f| find a narrow bracket of it first (22 leading key
 // bits); only members whose d_f lies within the rounding error of the bracket are
-// evaluated in FP64. Returns false where the bracket does not work out (many equal values, or
-// a spread that FP32 does not resolve around med): the caller selects on FP64 keys.
-template <int NT, class Val>
-__device__ bool block_mad(int nh, int k, bool even, double med, Val val, FitSmem &s, double *out) {
+// evaluated in FP64. The one before is mostly below the bracket (a slice of 2^-14), and then
+// found by one pass over the FP64 values: by d_f, two values on either side of a key's edge
+// may come in the wrong order. Returns false where the bracket does not work out (many equal
+// values, or a spread that FP32 does not resolve around med): the caller selects on FP64 keys.
+template <int NT, class Val, class Get>
+__device__ bool block_mad(int nh, int k, bool even, double med, Val val, Get getd, FitSmem &s, double *out) {
   const int t = threadIdx.x;
   const float mf = (float)med;
   auto getf = [&](int i, unsigned long long &key) {
@@ -252,51 +254,34 @@ __device__ bool block_mad(int nh, int k, bool even, double med, Val val, FitSmem
   if (t == 0) {
     s.cnt = 0;
     s.n = 0;
-    s.big = 0ULL;
   }
   __syncthreads();
   int below = 0;
-  unsigned long long mx = 0ULL;  // largest key below the bracket
 #pragma unroll 4
   for (int i = t; i < nh; i += NT) {
     const float x = val(i);
     if (!isfinite(x)) continue;
     const float d = fabsf(x - mf);
     if (d > fhi) continue;
-    if (d < flo && !(even && d > 0.0f && (float)(__float_as_uint(d) >> 9) + 2.0f > (float)top)) {
+    if (d < flo) {
       ++below;
       continue;
     }
     const double e = fabs(__dsub_rn((double)x, med));
-    const unsigned long long key = (unsigned long long)__double_as_longlong(e);
     if (e < lo) {
       ++below;
-      mx = key > mx ? key : mx;
     } else if (e <= hi) {
       const int at = atomicAdd(&s.cnt, 1);
-      if (at < kFitCand) s.cand[at] = key;
+      if (at < kFitCand) s.cand[at] = (unsigned long long)__double_as_longlong(e);
     }
   }
   below = __reduce_add_sync(0xffffffffu, below);
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = y > mx ? y : mx;
-  }
-  if ((t & 31) == 0) {
-    atomicAdd(&s.n, below);
-    atomicMax(&s.big, mx);
-  }
+  if ((t & 31) == 0) atomicAdd(&s.n, below);
   __syncthreads();
   const int m = s.cnt, r = k - s.n;
-  const unsigned long long prev = s.big;
   __syncthreads();
-  if (m > kFitCand || r < 0 || r >= m || (even && r == 0 && prev == 0ULL)) return false;
+  if (m > kFitCand || r < 0 || r >= m) return false;
   // rank r (and r - 1) of the m keys in shared memory: every thread ranks its own
-  if (t == 0) {
-    s.pre = 0ULL;
-    s.big = prev;
-  }
-  __syncthreads();
   for (int i = t; i < m; i += NT) {
     const unsigned long long key = s.cand[i];
     int less = 0, same = 0;
@@ -308,8 +293,11 @@ __device__ bool block_mad(int nh, int k, bool even, double med, Val val, FitSmem
     if (r > 0 && less <= r - 1 && r - 1 < less + same) s.big = key;
   }
   __syncthreads();
-  const double a = __longlong_as_double((long long)s.pre), b = __longlong_as_double((long long)s.big);
+  const unsigned long long ka = s.pre;
+  unsigned long long kb = s.big;
   __syncthreads();
+  if (even && r == 0) kb = block_prev_rank<NT>(nh, k, ka, getd, s);
+  const double a = __longlong_as_double((long long)ka), b = __longlong_as_double((long long)kb);
   *out = even ? 0.5 * (b + a) : a;
   return true;
 }
@@ -374,14 +362,14 @@ __global__ void __launch_bounds__(NT) k_fit_hist(const uint32_t *__restrict__ ho
       med = 0.5 * ((double)b + (double)a);
     }
   }
+  auto getd = [&](int i, unsigned long long &key) {
+    float x = rval(i);
+    if (!isfinite(x)) return false;
+    key = (unsigned long long)__double_as_longlong(fabs(__dsub_rn((double)x, med)));
+    return true;
+  };
   double mad;
-  if (!block_mad<NT>(nh, n / 2, !(n & 1), med, rval, s, &mad)) {
-    auto getd = [&](int i, unsigned long long &key) {
-      float x = rval(i);
-      if (!isfinite(x)) return false;
-      key = (unsigned long long)__double_as_longlong(fabs(__dsub_rn((double)x, med)));
-      return true;
-    };
+  if (!block_mad<NT>(nh, n / 2, !(n & 1), med, rval, getd, s, &mad)) {
     const unsigned long long ka = block_select<NT>(nh, n / 2, 64, getd, s);
     mad = __longlong_as_double((long long)ka);
     if (!(n & 1))

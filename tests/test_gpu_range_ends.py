@@ -193,3 +193,66 @@ def test_contexts_on_host_threads_with_different_bin_counts():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+# --------------------------------------------------- the fit's median and MAD, to the last bit
+def _mad(x):
+    """1.4826 median |x - median(x)| of the finite values, in FP64 as the fit defines it."""
+    x = np.sort(x[np.isfinite(x)].astype(np.float64))
+    n = len(x)
+    med = x[n // 2] if n & 1 else 0.5 * (x[n // 2 - 1] + x[n // 2])
+    d = np.sort(np.abs(x - med))
+    return 1.4826 * (d[n // 2] if n & 1 else 0.5 * (d[n // 2 - 1] + d[n // 2]))
+
+
+def _ratio_of(ctx, target, seed):
+    """A halo with f_l chosen such that R comes out as `target` to the last FP32 bit, with no
+    iterations of the fit: sigma_R is MAD' then. Returns (R, halo rows)."""
+    from paper_1902_01010_gb300 import Params
+
+    n = len(target)
+    rng = np.random.default_rng(seed)
+    pos = (np.round(rng.normal(0, 30000, (n, 3))).astype(np.int64) % L).astype(np.int32)
+    d = [_dev(pos), _dev(rng.normal(0, 0.4, (n, 3)).astype(np.float32)), None,
+         torch.zeros(n, dtype=torch.int32, device="cuda")]
+    P = Params.default(fit_iters=0)
+    ln_fl = np.zeros(n)
+    for _ in range(4):
+        d[2] = _dev(np.exp(ln_fl).astype(np.float32))
+        R, _, hs = ctx.outlier_ratio(d[0], d[1], d[2], d[3], P)
+        ctx.sync()
+        R = R.cpu().numpy()
+        if np.array_equal(R, target.astype(np.float32)):
+            break
+        ln_fl += target - R.astype(np.float64)
+    return R, hs.cpu().numpy()
+
+
+@pytest.mark.parametrize("n", [160, 161, 400, 1001, 4000, 16384, 20001, 40000])
+@pytest.mark.parametrize("centre,width", [(0.05, 0.4), (3.0, 4.0), (-20.0, 0.05), (0.0, 12.0)])
+def test_mad_is_exact(ctx, n, centre, width):
+    """Odd and even counts, with MADs well below and above 1 and far from the median's size."""
+    rng = np.random.default_rng(n)
+    R, hs = _ratio_of(ctx, rng.normal(centre, width, n), n)
+    assert hs[0, 4] == _mad(R)
+
+
+def test_mad_of_values_on_either_side_of_a_key_edge(ctx):
+    """An even count whose median lies half an ulp off the FP32 grid: of the two values next
+    below the middle distance, one below and one above the median, the FP32 distances have
+    the order that the exact ones have not."""
+    u = 2.0 ** -18                      # spacing of FP32 in [32, 64)
+    b = 32.0 + 2 * u                    # even mantissa: the median b + u/2 rounds down to it
+    edge, top = 0.75 - 2.0 ** -15, 0.75
+    up = lambda dist: b + dist
+    dn = lambda dist: b - dist
+    rng = np.random.default_rng(4)
+    grid = lambda x, g: np.round(x / g) * g
+    small = grid(rng.uniform(0.1, 0.6, 96), u)
+    big = grid(rng.uniform(1.2, 1.9, 99), u)
+    x = np.r_[b, b + u, up(edge), dn(edge - u / 2), up(top + 3 * u),
+              up(small[:48]), dn(small[48:]), up(big[:49]), dn(big[49:])]
+    assert len(x) == 200 and (x > b + u / 2).sum() == 100 and np.array_equal(x, x.astype(np.float32))
+    R, hs = _ratio_of(ctx, x, 1)
+    assert np.array_equal(R, x.astype(np.float32))
+    assert hs[0, 4] == _mad(R)
