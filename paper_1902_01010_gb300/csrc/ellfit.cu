@@ -20,6 +20,7 @@
 #include "halos.cuh"
 #include "vr_workspace.h"
 #include "background.cuh"
+#include "fit_bracket.h"
 
 namespace vr {
 
@@ -240,16 +241,12 @@ __device__ bool block_mad(int nh, int k, bool even, double med, Val val, Get get
   const float mf = (float)med;
   auto getf = [&](int i, unsigned long long &key) {
     const float x = val(i);
-    key = __float_as_uint(fabsf(x - mf)) >> 9;  // 22 bits
+    key = __float_as_uint(fabsf(x - mf)) >> kDistDrop;
     return (bool)isfinite(x);
   };
-  const uint32_t top = (uint32_t)block_select<NT>(nh, k, 22, getf, s);
-  if (top >= 0x3f8000u >> 1) return false;  // infinite distance
-  const double blo = (double)__uint_as_float(top << 9), bhi = (double)__uint_as_float((top + 1u) << 9);
-  // |d_f - d|: the rounding of med and of the difference
-  const double err = 1.2e-7 * (fabs(med) + bhi);
-  const double lo = blo - 4.0 * err, hi = bhi + 4.0 * err;  // holds rank k, and k - 1 unless alone
-  if (!(err < 0.25 * (bhi - blo))) return false;
+  const uint32_t top = (uint32_t)block_select<NT>(nh, k, kDistBits, getf, s);
+  double lo, hi, err;  // [lo, hi] holds rank k
+  if (!dist_bracket(top, med, &lo, &hi, &err)) return false;
   const float flo = (float)(lo - 4.0 * err), fhi = (float)(hi + 4.0 * err);
   if (t == 0) {
     s.cnt = 0;
