@@ -412,8 +412,9 @@ vr_status vr_autotune(vr_ctx *ctx, int enable);
  * shapes agree. Errors: VR_ERR_INVALID_ARG for an index out of range. */
 vr_status vr_tuning_force(vr_ctx *ctx, int velden_shape, int link_shape);
 
-/* Writes a JSON object with the candidate shapes, the shape in use per bin and the
- * measured milliseconds (-1 where not measured) into buf (len bytes, NUL-terminated).
+/* Writes a JSON object with the candidate shapes, the shape in use per bin (forced, tuned,
+ * or the one that the bin's last launch took by its size; 0 before any) and the measured
+ * milliseconds (-1 where not measured) into buf (len bytes, NUL-terminated).
  * Errors: VR_ERR_INVALID_ARG if buf is too small. */
 vr_status vr_tuning_report(const vr_ctx *ctx, char *buf, size_t len);
 

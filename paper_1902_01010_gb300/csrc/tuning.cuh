@@ -8,6 +8,7 @@ namespace vr {
 
 // f_l launches by halo size (members): above 65536, (4096, 65536], (N_se, 4096].
 constexpr int kVBins = 3;
+static_assert(sizeof(vr_ctx::vshape_last) == kVBins * sizeof(int), "one entry per bin");
 constexpr uint32_t kVBinEdge0 = 65536u, kVBinEdge1 = 4096u;
 
 // f_l kernel shapes: candidates computed side by side, register cap, warps per block.
@@ -32,9 +33,12 @@ struct Tuning {
 };
 
 // Shape index for f_l bin k / the linker under the context's tuning state. Untuned f_l
-// launches of many buckets take 2 warps per block, whose places are free again sooner (256^3 box,
-// 150,000 buckets: 33.3 ms with 4 warps, 32.6 with 2; a catalogue of 180,000: 23.2 and 22.7); of
-// few buckets 4, of which more start at once (1M particles, 8,900 buckets: 3.39 and 3.44).
+// launches of many buckets take 2 warps per block, whose places are free again sooner, of few
+// buckets 4, of which more start at once. Call with 2 warps against 4, three seeds each, by
+// buckets (the spread of repeated calls in brackets): 2,400 -1.2 to +0.3 % (1.5), 11,000 to
+// 12,500 -2.4 to +2.0 (3), 21,000 to 28,000 -1.3 to +0.9 (4), 32,000 -0.8 to -1.0 (0.6), 38,000
+// -1.0 to -1.2 (0.5), 47,000 -1.1 to -1.4 (0.2), 65,000 -1.2 to -1.5 (0.3), 187,000 (256^3 box,
+// 36.9 -> 36.3 ms) -1.5 (0.1), 210,000 (catalogue, N_se 64) -1.9 (0.1).
 constexpr int64_t kVManyBuckets = 32768;
 constexpr int kVShapeMany = 2;
 inline int vshape_for(const vr_ctx *ctx, int k, int64_t buckets = 0) {
@@ -42,6 +46,14 @@ inline int vshape_for(const vr_ctx *ctx, int k, int64_t buckets = 0) {
   if (t && t->force_v >= 0) return t->force_v;
   if (t && t->vtuned[k]) return t->vshape[k];
   return buckets >= kVManyBuckets ? kVShapeMany : 0;
+}
+// True when bin k's f_l shape follows from its launch's size: neither forced nor tuned.
+inline bool vshape_by_size(const vr_ctx *ctx, int k) {
+  return !ctx->tune || (ctx->tune->force_v < 0 && !ctx->tune->vtuned[k]);
+}
+// The f_l shape in use for bin k: forced, tuned, or what its last launch took by its size.
+inline int vshape_in_use(const vr_ctx *ctx, int k) {
+  return vshape_by_size(ctx, k) ? ctx->vshape_last[k] : vshape_for(ctx, k);
 }
 inline int lshape_for(const vr_ctx *ctx) {
   const Tuning *t = ctx ? ctx->tune : nullptr;

@@ -1041,6 +1041,8 @@ vr_status run_velden(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &a
       while (k + 1 < kVBins && !(k == 0 && ev_big) &&
              (p->nv > 32 || (!vmeasure(ctx, k + 1) && vshape_for(ctx, k + 1, nbpad) == sh)))
         ++k;
+      for (int j = 0; j < kVBins; ++j)
+        if (hi[j] > lo[j] && lo[j] >= first && hi[j] <= hi[k] && vshape_by_size(ctx, j)) ctx->vshape_last[j] = sh;
       VR_CUDA(ctx, big(sh, first, hi[k]));
       VR_LAUNCHED(ctx, "k_velden_big");
     }

@@ -304,6 +304,7 @@ vr_status vr_autotune(vr_ctx *ctx, int enable) {
   for (int k = 0; k < kVBins; ++k) {
     t->vtuned[k] = 0;
     t->vshape[k] = 0;
+    ctx->vshape_last[k] = 0;
   }
   t->ltuned = 0;
   t->lshape = 0;
@@ -334,7 +335,7 @@ vr_status vr_tuning_report(const vr_ctx *ctx, char *buf, size_t len) {
   }
   o += "], \"chosen\": [";
   for (int k = 0; k < kVBins; ++k) {
-    snprintf(tmp, sizeof(tmp), "%s%d", k ? ", " : "", vshape_for(ctx, k));
+    snprintf(tmp, sizeof(tmp), "%s%d", k ? ", " : "", vshape_in_use(ctx, k));
     o += tmp;
   }
   o += "], \"measured\": [";

@@ -43,6 +43,7 @@ struct vr_ctx {
   cudaStream_t side2;       // third stream: the cell-tree build beside the f_l stage
   cudaEvent_t ev_fork2, ev_join2;
   cudaEvent_t ev_flbig, ev_tail;  // f_l of the largest halos done; their R and fit done
+  int vshape_last[3];       // f_l shape that each halo-size bin's last launch took by its size (vr_tuning_report)
   int log_level;            // vr_set_log_level: 0 silent, 1 errors, 2 errors and calls
 };
 

@@ -256,3 +256,29 @@ def test_mad_of_values_on_either_side_of_a_key_edge(ctx):
     R, hs = _ratio_of(ctx, x, 1)
     assert np.array_equal(R, x.astype(np.float32))
     assert hs[0, 4] == _mad(R)
+
+
+# -------------------------------------------------------- the shape that a launch takes
+def test_tuning_report_names_the_shapes_of_untuned_launches():
+    """1.1 M members in one halo are more than 32,768 buckets, 5,000 are few: each takes the
+    shape of its size, and the report names it; a forced shape is named instead."""
+    from paper_1902_01010_gb300 import Context
+
+    c = Context(0)
+    assert c.tuning_report()["f_l"]["chosen"] == [0, 0, 0]
+    rng = np.random.default_rng(8)
+
+    def call(n):
+        pos = _dev((np.round(rng.normal(0, 60000, (n, 3))).astype(np.int64) % L).astype(np.int32))
+        c.velden(pos, _dev(rng.normal(0, 80, (n, 3)).astype(np.float32)),
+                 torch.zeros(n, dtype=torch.int32, device="cuda"))
+        c.sync()
+        rep = c.tuning_report()["f_l"]
+        return [rep["shapes"][k]["warps"] for k in rep["chosen"]]
+
+    assert call(1_100_000) == [2, 4, 4]
+    assert call(5000) == [2, 4, 4]  # the middle bin's; the first had no launch
+    c.tuning_force(1, -1)
+    assert call(5000) == [8, 8, 8]
+    c.tuning_force(-1, -1)
+    assert call(5000) == [2, 4, 4]
