@@ -254,25 +254,68 @@ __device__ __forceinline__ void core_moments(
   }
 }
 
-// A cluster per core. The sums are FP64 (some 45 operations a member, of which an SM does two
-// lanes a cycle) over the whole halo's slots, twice, so the blocks share the halos of kTeamHalo
-// members and more; a smaller one is left to the first block (128^3 box, six
-// launches: 2.91 -> 2.01 ms). With l >= 0 only
-// cores that are active at level l are recomputed, in halos that grow.
+// The sums are FP64 (some 45 operations a member, of which an SM does two lanes a cycle) over
+// the whole halo's slots, twice. A cluster of kCoreTeam blocks shares a core whose halo is more
+// than half an SM's share of all cores' slots, a block takes each of the others, side by side on
+// two streams. The reductions cost a block some 11 us whatever its part of the halo, and a block
+// of the cluster form (255 registers a thread, 128 in the other) has an SM to itself, so clusters
+// for cores that fill the chip without them cost a multiple (whole calls with clusters for every
+// halo, or for all of 4,096 members and more, and by this rule: 20,000 halos of 40 members 86.9
+// and 21.6 ms, of 200 members 195.6 and 52.4, 200 halos of 5,000 11.8 and 5.0; boxes of 128^3
+// 8.17 and 7.78, of 200^3 20.5 and 19.2; with the line at a whole share, an eighth of one, or the
+// two launches in a row 8.0 to 8.1 and 19.1 to 19.4). By the rule at most two clusters per SM have
+// work, so their grid needs no count from the device.
 constexpr int kCoreTeam = 8;
-constexpr uint32_t kTeamHalo = 4096;
-__global__ void __launch_bounds__(kCT) __cluster_dims__(kCoreTeam, 1, 1) k_cg_moments(
+constexpr uint32_t kTeamHalo = 4096;  // fewer members are not worth a team
+constexpr int kMaxTeams = 1024;       // entries of the list of the clusters' cores
+
+struct CoreTeams {
+  unsigned long long *slots;  // slots of all cores' halos, a halo counted once per core
+  int32_t *list;              // cores that clusters take, their number in list[-1]
+  int max;                    // twice the SMs: cores of more than 1 / max of all slots have a team
+};
+
+__device__ __forceinline__ bool core_has_team(uint32_t nh, const CoreTeams &ct) {
+  return nh >= kTeamHalo && (unsigned long long)nh * ct.max >= *ct.slots;
+}
+
+__global__ void k_cg_slots_sum(int64_t K, CoreTab t, const uint32_t *__restrict__ hoff, CoreTeams ct) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned long long nh = k < K ? hoff[t.halo[k] + 1] - hoff[t.halo[k]] : 0;
+  for (int o = 16; o; o >>= 1) nh += __shfl_down_sync(0xffffffffu, nh, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(ct.slots, nh);
+}
+
+__global__ void k_cg_teams(int64_t K, CoreTab t, const uint32_t *__restrict__ hoff, CoreTeams ct) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= K || !core_has_team(hoff[t.halo[k] + 1] - hoff[t.halo[k]], ct)) return;
+  ct.list[atomicAdd(&ct.list[-1], 1)] = (int32_t)k;  // at most ct.max of them
+}
+
+// With l >= 0 only cores that are active at level l are recomputed, in halos that grow.
+__device__ __forceinline__ bool core_wanted(const CoreTab &t, int k, int l, const int *hgrow) {
+  return l < 0 || (t.alive[k] && (t.prim[k] || t.level[k] >= l) && hgrow[t.halo[k]]);
+}
+
+__global__ void __launch_bounds__(kCT) k_cg_moments(
     const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ pre, const int4 *__restrict__ u,
     const float4 *__restrict__ v, const int32_t *__restrict__ gc, const int32_t *__restrict__ searched,
-    CoreTab t, int l, const int *__restrict__ hgrow, int clean, double beta_c) {
-  const int k = (int)(blockIdx.x / kCoreTeam), part = (int)(blockIdx.x % kCoreTeam);
-  if (l >= 0 && !(t.alive[k] && (t.prim[k] || t.level[k] >= l) && hgrow[t.halo[k]])) return;
-  if (hoff[t.halo[k] + 1] - hoff[t.halo[k]] >= kTeamHalo) {
-    core_moments<kCoreTeam>(k, part, hoff, pre, u, v, gc, searched, t, clean, beta_c);
-    cg::this_cluster().sync();  // the others may still read this block's sums
-  } else if (part == 0) {
-    core_moments<1>(k, 0, hoff, pre, u, v, gc, searched, t, clean, beta_c);
-  }
+    CoreTab t, int l, const int *__restrict__ hgrow, int clean, double beta_c, CoreTeams ct) {
+  const int k = (int)blockIdx.x;
+  if (!core_wanted(t, k, l, hgrow) || core_has_team(hoff[t.halo[k] + 1] - hoff[t.halo[k]], ct)) return;
+  core_moments<1>(k, 0, hoff, pre, u, v, gc, searched, t, clean, beta_c);
+}
+
+__global__ void __launch_bounds__(kCT) __cluster_dims__(kCoreTeam, 1, 1) k_cg_moments_team(
+    const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ pre, const int4 *__restrict__ u,
+    const float4 *__restrict__ v, const int32_t *__restrict__ gc, const int32_t *__restrict__ searched,
+    CoreTab t, int l, const int *__restrict__ hgrow, int clean, double beta_c, CoreTeams ct) {
+  const int i = (int)(blockIdx.x / kCoreTeam), part = (int)(blockIdx.x % kCoreTeam);
+  if (i >= ct.list[-1]) return;  // the same for the whole cluster, as below
+  const int k = ct.list[i];
+  if (!core_wanted(t, k, l, hgrow)) return;
+  core_moments<kCoreTeam>(k, part, hoff, pre, u, v, gc, searched, t, clean, beta_c);
+  cg::this_cluster().sync();  // the others may still read this block's sums
 }
 
 // Members of dropped cores return to the untagged background; halos that keep a
@@ -348,6 +391,8 @@ size_t coregrow_bytes(int64_t n, int nmin) {
   ar.take<double>(21 * kmax);
   ar.take<double>(21 * kmax);
   ar.take<unsigned long long>(1);
+  ar.take<unsigned long long>(1);      // CoreTeams
+  ar.take<int32_t>(kMaxTeams + 1);
   return ar.off + scan_scratch_bytes<uint32_t>(n + 1) + 4096;
 }
 
@@ -388,25 +433,46 @@ vr_status run_core_grow(vr_ctx *ctx, const HaloSeg &g, const vr_core_params *cp,
   t.mean = ar.take<double>(6 * K);
   t.S = ar.take<double>(21 * K);
   t.L = ar.take<double>(21 * K);
+  CoreTeams ct;
+  ct.slots = ar.take<unsigned long long>(1);
+  int32_t *teams = ar.take<int32_t>(kMaxTeams + 1);
+  ct.list = teams + 1;
+  ct.max = 2 * ctx->sm_count < kMaxTeams ? 2 * ctx->sm_count : kMaxTeams;
   if (!ar.ok()) return set_error(ctx, VR_ERR_WORKSPACE_TOO_SMALL, "workspace too small");
   k_cg_table<<<grid_for(NHP, T), T, 0, s>>>(g.hid, g.v, NHP, core, level, pre, ex.prim, ex.last, t,
                                             cid_of);
   VR_LAUNCHED(ctx, "k_cg_table");
   k_cg_slots<<<grid_for(NHP, T), T, 0, s>>>(g.v, NHP, core, cid_of, gc);
   VR_LAUNCHED(ctx, "k_cg_slots");
+  VR_CUDA(ctx, cudaMemsetAsync(ct.slots, 0, sizeof(unsigned long long), s));
+  VR_CUDA(ctx, cudaMemsetAsync(teams, 0, sizeof(int32_t), s));
+  k_cg_slots_sum<<<grid_for(K, T), T, 0, s>>>(K, t, g.hoff, ct);
+  VR_LAUNCHED(ctx, "k_cg_slots_sum");
+  k_cg_teams<<<grid_for(K, T), T, 0, s>>>(K, t, g.hoff, ct);
+  VR_LAUNCHED(ctx, "k_cg_teams");
+  const unsigned nteams = (unsigned)(K < ct.max ? K : ct.max);
+  auto moments = [&](int l, int clean, double beta_c) -> vr_status {
+    timer_begin(ctx, "core_grow", s);
+    VR_CUDA(ctx, cudaEventRecord(ctx->ev_fork, s));
+    VR_CUDA(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+    k_cg_moments_team<<<kCoreTeam * nteams, kCT, 0, ctx->side>>>(g.hoff, pre, g.u, g.v, gc, ex.searched, t, l,
+                                                                 hgrow, clean, beta_c, ct);
+    VR_LAUNCHED(ctx, "k_cg_moments_team");
+    VR_CUDA(ctx, cudaEventRecord(ctx->ev_join, ctx->side));
+    k_cg_moments<<<(unsigned)K, kCT, 0, s>>>(g.hoff, pre, g.u, g.v, gc, ex.searched, t, l, hgrow, clean, beta_c,
+                                             ct);
+    VR_LAUNCHED(ctx, "k_cg_moments");
+    VR_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_join, 0));
+    timer_end(ctx, "core_grow", s);
+    return VR_OK;
+  };
   // the cores as found, and the cleaning
-  VR_TIMED(ctx, "core_grow", s, k_cg_moments<<<(unsigned)(kCoreTeam * K), kCT, 0, s>>>(
-      g.hoff, pre, g.u, g.v, gc, ex.searched, t, -1, hgrow, 1, gp->beta_c));
-  VR_LAUNCHED(ctx, "k_cg_moments");
+  if ((st = moments(-1, 1, gp->beta_c)) != VR_OK) return st;
   VR_CUDA(ctx, cudaMemsetAsync(hgrow, 0, H * sizeof(int), s));
   k_cg_drop<<<grid_for(NHP, T), T, 0, s>>>(NHP, g.hid, t, gc, hgrow);
   VR_LAUNCHED(ctx, "k_cg_drop");
   for (int l = cp->n_loop - 1; l >= 0; --l) {
-    if (gp->mode == 2) {
-      VR_TIMED(ctx, "core_grow", s, k_cg_moments<<<(unsigned)(kCoreTeam * K), kCT, 0, s>>>(
-          g.hoff, pre, g.u, g.v, gc, ex.searched, t, l, hgrow, 0, 0.0));
-      VR_LAUNCHED(ctx, "k_cg_moments");
-    }
+    if (gp->mode == 2 && (st = moments(l, 0, 0.0)) != VR_OK) return st;
     VR_TIMED(ctx, "core_grow", s, k_cg_assign<<<grid_for(NHP, T), T, 0, s>>>(
         NHP, g.hid, g.hoff, pre, g.u, g.v, ex.searched, hgrow, t, l, gp->mode, gc));
     VR_LAUNCHED(ctx, "k_cg_assign");

@@ -282,3 +282,27 @@ def test_tuning_report_names_the_shapes_of_untuned_launches():
     assert call(5000) == [8, 8, 8]
     c.tuning_force(-1, -1)
     assert call(5000) == [2, 4, 4]
+
+
+# ------------------------------------------- core moments: clusters for large halos' cores
+@pytest.mark.parametrize("small", [300, 5000])
+def test_core_moments_of_many_halos_beside_a_large_one(ctx, small):
+    """300 halos of two cores, whose moments a block takes each (also where a halo alone in the
+    box, of 5,000 members, would have a cluster), and one of 13,000 members, which has."""
+    from test_gpu_coregrow import _check
+
+    rng = np.random.default_rng(small)
+    g = np.stack(np.meshgrid(*[np.arange(5)] * 3, indexing="ij"), -1).reshape(-1, 3) * 500
+    sizes, pos, vel, lab = [13000] + 300 * [small], [], [], []
+    for n in sizes:
+        base = np.array([100000, 100000, 100000])
+        d = rng.normal(size=(n - 2 * len(g), 3))
+        d = d / np.linalg.norm(d, axis=1)[:, None] * rng.uniform(9000, 90000, (len(d), 1))
+        pos += [g + base, g + base + [3500, 0, 0], np.round(base + [3250, 1500, 1500] + d)]
+        vel += [rng.normal(0, 0.3, size=(len(g), 3)) + [s, 0, 0] for s in (200, -200)]
+        vel.append(rng.normal(0, 60, size=(len(d), 3)))
+        lab.append(np.full(n, sum(map(len, lab))))
+    pos, vel = np.vstack(pos).astype(np.int32), np.vstack(vel).astype(np.float32)
+    core, grown, kept = _check(ctx, pos, vel, np.concatenate(lab).astype(np.int32), None, 700.0,
+                               halos=[0, 1, 150, 300], f_c=0.005)
+    assert kept == 2 * len(sizes) and (grown != core).any()
