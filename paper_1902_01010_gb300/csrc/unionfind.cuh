@@ -22,6 +22,16 @@ __device__ __forceinline__ int uf_find(int *parent, int x) {
   }
 }
 
+// The root of x without halving its path: for kernels in which many threads find the same x, whose
+// stores to one word would hold up each other's loads.
+__device__ __forceinline__ int uf_root(const int *parent, int x) {
+  while (true) {
+    const int p = uf_load(parent, x);
+    if (p == x) return x;
+    x = p;
+  }
+}
+
 __device__ __forceinline__ void uf_unite(int *parent, int a, int b) {
   while (true) {
     a = uf_find(parent, a);

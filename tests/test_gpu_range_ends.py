@@ -306,3 +306,19 @@ def test_core_moments_of_many_halos_beside_a_large_one(ctx, small):
     core, grown, kept = _check(ctx, pos, vel, np.concatenate(lab).astype(np.int32), None, 700.0,
                                halos=[0, 1, 150, 300], f_c=0.005)
     assert kept == 2 * len(sizes) and (grown != core).any()
+
+
+# ---------------------------------------------- 3D FOF: thousands of particles a sub-cell
+@pytest.mark.parametrize("n,spread,T", [(40000, 100, 5000 ** 2), (33, 1, 9), (50000, 2000, 5000 ** 2),
+                                        (4097, 300, 900 ** 2)])
+def test_fof_crowded_sub_cells(ctx, n, spread, T):
+    """A clump across the corner where eight sub-cells (and the box's periodic edges) meet, a
+    second one out of reach, and single particles between sub-cells of many."""
+    rng = np.random.default_rng(n)
+    p = np.concatenate([rng.normal(0, spread, (n, 3)), rng.normal(300000, spread, (n // 2, 3)),
+                        rng.integers(0, L, (200, 3))])
+    pos = (np.round(p).astype(np.int64) % L).astype(np.int32)
+    pos = pos[rng.permutation(len(pos))]
+    lab = ctx.fof3d(_dev(pos), T)
+    ctx.sync()
+    assert np.array_equal(lab.cpu().numpy(), oracle.fof3d(pos, T))
