@@ -256,8 +256,11 @@ __device__ __forceinline__ void frame_len(const LinkC &c, float4 q, float &s, fl
 // The predicate for members a and b: fa, fb positions as FP32 (whole numbers below 2^23,
 // so every difference is exact), qa, qb velocities, (s, r) from frame_len (used with
 // V_r / Theta_op only). FP32 errors: q below 8 * 2^-24 < 5e-7 relative, decided outside
-// [1 - 1e-5, 1 + 1e-5]; the V_r and Theta_op tests within ra + rb. NaN settles nothing and
-// goes to FP64.
+// [1 - 1e-5, 1 + 1e-5]; the V_r and Theta_op tests within e = ra + rb < 0.5, a first-order bound
+// with room: for pairs that FP64 links (at most 90 degrees apart) the rounding of the frame moves
+// the ratio of the two lengths by at most 0.93 e, the cosine by 0.42 e (worst over 2e8 draws of
+// frames, pairs at the thresholds and V_r of 1 to 30), and a pair beyond 90 degrees that V_r
+// rejects wrongly is rejected all the same. NaN settles nothing and goes to FP64.
 __device__ __forceinline__ bool pair_link(const LinkC &c, float4 fa, float4 qa, float sa, float ra,
                                           float4 fb, float4 qb, float sb, float rb) {
   const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;

@@ -322,3 +322,33 @@ def test_fof_crowded_sub_cells(ctx, n, spread, T):
     lab = ctx.fof3d(_dev(pos), T)
     ctx.sync()
     assert np.array_equal(lab.cpu().numpy(), oracle.fof3d(pos, T))
+
+
+# ------------------------------------------------ 6D links far from the halo frame's origin
+@pytest.mark.parametrize("bulk", [3000.0, 1.0e6])
+@pytest.mark.parametrize("v_ratio,theta,use_lv", [(2.0, 0.314, 1), (1.2, 0.9, 0), (1.05, 1.5, 0), (5.0, 1.57, 1)])
+def test_links_with_a_bulk_velocity_far_above_the_dispersion(ctx, bulk, v_ratio, theta, use_lv):
+    """Velocities a few FP32 spacings from a halo velocity that lies between them: the rounding
+    of the frame is a good part of every member's velocity in it."""
+    from paper_1902_01010_gb300 import Params
+
+    rng = np.random.default_rng(int(bulk))
+    ulp = float(np.spacing(np.float32(bulk)))
+    n = 1500
+    pos = (rng.integers(0, 9, (n, 3)) * 500 + 3000).astype(np.int32)
+    k = np.where(rng.random((n, 1)) < 0.5, rng.integers(-9, 10, (n, 3)), rng.integers(-60, 61, (n, 3)))
+    vel = (bulk + k * ulp).astype(np.float32)
+    ell = np.where(rng.random(n) < 0.8, 3.0, 1.0).astype(np.float32)
+    for frac in ([0.5, 0.5, 0.5], [0.49, -0.5, 0.26], [0.0, 0.5, -0.37]):
+        hs = np.zeros((1, 12))
+        hs[0, :3] = [0, n, 1]
+        hs[0, 5:8] = bulk + np.array(frac) * ulp
+        hs[0, 9], hs[0, 10] = 500.0 ** 2 * 1.5, (14 * ulp) ** 2
+        P = Params.default(nsearch_min=20, nmin=2, use_lv=use_lv, v_ratio=v_ratio, theta_op=theta)
+        got = ctx.fof6d(_dev(pos), _dev(vel), _dev(ell), _dev(np.zeros(n, np.int32)), _dev(hs), P)
+        ctx.sync()
+        m = np.arange(n)
+        ref = oracle.fof6d_halo(oracle.unwrap(pos, m), vel, m, (ell >= 2.5).astype(np.uint8),
+                                hs[0, [9, 10, 5, 6, 7]], v_ratio, theta, use_lv=use_lv, nmin=2)
+        assert np.array_equal(got.cpu().numpy(), ref)
+        assert len(np.unique(ref)) > 2
