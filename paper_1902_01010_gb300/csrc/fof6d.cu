@@ -718,13 +718,18 @@ cudaError_t link_tiles(const Cands &C, int64_t t0, int64_t t1, int warps, const 
 
 // ------------------------------------------------------- two-stage linking kernels
 
-// Stage-1 label of each candidate and stage-1 group sizes (indexed by label).
+// Stage-1 label of each candidate and stage-1 group sizes (indexed by label; one of n or more
+// raises an error and counts as none).
 __global__ void k_grow_tags(const float4 *__restrict__ cv, int64_t nc,
-                            const int32_t *__restrict__ label6, int *__restrict__ tag,
-                            int *__restrict__ n0) {
+                            const int32_t *__restrict__ label6, int64_t n, int *__restrict__ tag,
+                            int *__restrict__ n0, DevStatus *st) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nc) return;
-  const int t = label6[__float_as_int(cv[c].w)];
+  int t = label6[__float_as_int(cv[c].w)];
+  if (t >= n) {
+    raise_error(st, VR_ERR_INVALID_ARG, 6);
+    t = -1;
+  }
   tag[c] = t;
   if (t >= 0) atomicAdd(&n0[t], 1);
 }
@@ -1007,7 +1012,7 @@ vr_status run_grow(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, const vr_g
   const int T = 256;
   VR_CUDA(ctx, cudaMemsetAsync(n0, 0, n * sizeof(int), s));
   VR_CUDA(ctx, cudaMemsetAsync(best, 0, nc * sizeof(unsigned long long), s));
-  k_grow_tags<<<grid_for(nc, T), T, 0, s>>>(C.cv, nc, label6, tag, n0);
+  k_grow_tags<<<grid_for(nc, T), T, 0, s>>>(C.cv, nc, label6, n, tag, n0, ctx->d_status);
   VR_LAUNCHED(ctx, "k_grow_tags");
   const double vr = p->v_ratio * gp->gamma_vr, ct = cos(p->theta_op * gp->gamma_theta);
   const double vr2 = vr * vr, cos2 = ct * ct;

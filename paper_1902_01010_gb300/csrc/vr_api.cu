@@ -149,6 +149,7 @@ vr_status read_status(vr_ctx *ctx, cudaStream_t s, DevStatus *out) {
       case 3: what = "background cell tree exceeded its depth bound"; break;
       case 4: what = "a 3D label lies outside [0, n)"; break;
       case 5: what = "link-count table of the two-stage linking is full"; break;
+      case 6: what = "a stage-1 label of the two-stage linking is n or more"; break;
       default: break;
     }
     // clear for the next call

@@ -352,3 +352,31 @@ def test_links_with_a_bulk_velocity_far_above_the_dispersion(ctx, bulk, v_ratio,
                                 hs[0, [9, 10, 5, 6, 7]], v_ratio, theta, use_lv=use_lv, nmin=2)
         assert np.array_equal(got.cpu().numpy(), ref)
         assert len(np.unique(ref)) > 2
+
+
+@pytest.mark.parametrize("bad", [600, (1 << 31) - 1])
+def test_stage_1_label_out_of_range_is_refused(ctx, bad):
+    """A label6 of n or more among the groups to grow: VR_ERR_INVALID_ARG, and the next call works."""
+    from paper_1902_01010_gb300 import VrError
+
+    rng = np.random.default_rng(5)
+    n = 600
+    pos, vel = _dev(rng.integers(0, 4000, (n, 3)).astype(np.int32)), _dev(rng.normal(0, 50, (n, 3)).astype(np.float32))
+    ell, lab = _dev(np.full(n, 3.0, np.float32)), torch.zeros(n, dtype=torch.int32, device="cuda")
+    hs = np.zeros((1, 12))
+    hs[0, :3] = [0, n, 1]
+    hs[0, 9], hs[0, 10] = 300.0 ** 2, 40.0 ** 2
+    good = ctx.fof6d(pos, vel, ell, lab, _dev(hs))
+    ctx.sync()
+    want = good.clone()
+    ctx.grow_groups(pos, vel, ell, lab, _dev(hs), want)
+    l6 = good.clone()
+    l6[123] = bad
+    with pytest.raises(VrError) as e:
+        ctx.grow_groups(pos, vel, ell, lab, _dev(hs), l6)
+        ctx.sync()
+    assert e.value.code == 1 and "stage-1 label" in str(e.value)
+    got = good.clone()
+    ctx.grow_groups(pos, vel, ell, lab, _dev(hs), got)
+    ctx.sync()
+    assert torch.equal(got, want)
