@@ -34,6 +34,7 @@
 
 #include <vector>
 
+#include "boxparts.cuh"
 #include "halos.cuh"
 #include "tuning.cuh"
 #include "vr_workspace.h"
@@ -499,52 +500,11 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     if (r2 >= (1LL << 41)) raise_error(st, VR_ERR_UNSUPPORTED, 1);
     return;
   }
-  // Two parts of the query bucket: where the curve jumps, its particles lie in two clumps, and
-  // one box would reach everything between them (in a halo of 564 k members one bucket
-  // tested 27,000 others one by one for 437 to visit: 25 M cycles, 13 ms, a third of the whole
-  // launch; the longest warp of any is 9 M cycles with two parts).
-  // Boxes of the particles up to each lane and from each lane on; the cut is where the two
-  // volumes are least, each extent with an eighth of the largest one added.
-  int cut = 31;
-  {
-    int4 alo = q, ahi = q, zlo = q, zhi = q;  // lanes beyond the bucket repeat its first particle
-    const int last = (int)(qe - qs) - 1;
-    auto from = [&](int4 a, int src) {
-      return make_int4(__shfl_sync(FULL, a.x, src), __shfl_sync(FULL, a.y, src), __shfl_sync(FULL, a.z, src), 0);
-    };
-    auto join = [](int4 &lo, int4 &hi, int4 l, int4 h) {
-      lo.x = min(lo.x, l.x); lo.y = min(lo.y, l.y); lo.z = min(lo.z, l.z);
-      hi.x = max(hi.x, h.x); hi.y = max(hi.y, h.y); hi.z = max(hi.z, h.z);
-    };
-    for (int o = 1; o < 32; o <<= 1) {
-      const int4 al = from(alo, lane - o), ah = from(ahi, lane - o), zl = from(zlo, lane + o), zh = from(zhi, lane + o);
-      if (lane >= o) join(alo, ahi, al, ah);
-      if (lane + o <= last) join(zlo, zhi, zl, zh);
-    }
-    const float m = 0.125f * (float)max(qhi.x - qlo.x, max(qhi.y - qlo.y, qhi.z - qlo.z));
-    auto vol = [&](int4 l, int4 h) {
-      return ((float)(h.x - l.x) + m) * ((float)(h.y - l.y) + m) * ((float)(h.z - l.z) + m);
-    };
-    const int4 nlo = from(zlo, lane + 1), nhi = from(zhi, lane + 1);
-    float best = lane < last ? vol(alo, ahi) + vol(nlo, nhi) : __int_as_float(0x7f800000);
-    int at = lane;
-    for (int o = 16; o; o >>= 1) {
-      const float ob = __shfl_xor_sync(FULL, best, o);
-      const int oa = __shfl_xor_sync(FULL, at, o);
-      if (ob < best || (ob == best && oa < at)) {
-        best = ob;
-        at = oa;
-      }
-    }
-    cut = at;  // 0 for a single particle, whose second part has no lane that wants anything
-    if (lane == at) {
-      sm.qlo[0] = alo;
-      sm.qhi[0] = ahi;
-      sm.qlo[1] = last > 0 ? nlo : alo;
-      sm.qhi[1] = last > 0 ? nhi : ahi;
-    }
-    __syncwarp();
-  }
+  // Two parts of the query bucket (a bucket whose box spanned a jump of the curve, in a halo of
+  // 564 k members, tested 27,000 others one by one for 437 to visit: 25 M cycles, 13 ms, a third of
+  // the whole launch; the longest warp of any is 9 M cycles with two parts).
+  const int cut = box_parts(q, (int)(qe - qs) - 1, qlo, qhi, sm.qlo, sm.qhi);
+  __syncwarp();
   // Candidate buckets are enumerated on the fly in every pass: super-bucket boxes, then
   // bucket boxes, against the query bucket's box grown by the largest per-lane bound;
   // f(bucket index) is called warp-uniformly for every bucket that passes.

@@ -380,3 +380,47 @@ def test_stage_1_label_out_of_range_is_refused(ctx, bad):
     ctx.grow_groups(pos, vel, ell, lab, _dev(hs), got)
     ctx.sync()
     assert torch.equal(got, want)
+
+
+# ------------------------------------- 6D links in flat, elongated and clumped-up halos
+@pytest.mark.parametrize("shape", ["line", "plane", "filament", "two clumps", "duplicates"])
+@pytest.mark.parametrize("n", [33, 1000, 5000])
+def test_links_in_flat_and_elongated_halos(ctx, shape, n):
+    """Halos that fill few cells of their bounding cube, where a tile of 32 members may lie on a
+    jump of the curve: the field 6DFOF, and the two-stage linking of its smaller groups."""
+    from paper_1902_01010_gb300 import GrowParams, Params
+
+    rng = np.random.default_rng(n)
+    z = np.zeros(n)
+    p = {"line": np.stack([rng.integers(0, 2 * n, n), z, z], 1),
+         "plane": np.stack([rng.integers(0, 9000, n), rng.integers(0, 9000, n), z], 1),
+         "filament": np.stack([rng.integers(0, 3 * n, n), rng.normal(0, 300, n), rng.normal(0, 300, n)], 1),
+         "two clumps": rng.normal(0, 500, (n, 3)) + rng.choice([0, 300000], (n, 1)),
+         "duplicates": np.repeat(rng.integers(0, 5000, (n // 7 + 1, 3)), 7, 0)[:n]}[shape]
+    pos = ((np.round(p).astype(np.int64) + 1000) % L).astype(np.int32)[rng.permutation(n)]
+    vel = rng.normal(0, 80, (n, 3)).astype(np.float32)
+    lab = np.zeros(n, np.int32)
+    P = Params.default(nsearch_min=20, nmin=4)
+    got, hs = ctx.fof6d_field(_dev(pos), _dev(vel), _dev(lab), 400.0, 1.25, P)
+    ctx.sync()
+    m = np.arange(n)
+    up = oracle.unwrap(pos, m)
+    row = hs[0].cpu().numpy()
+    ref = oracle.fof6d_halo(up, vel, m, np.ones(n, np.uint8), row[[9, 10, 5, 6, 7]], use_vt=0, nmin=4)
+    assert np.array_equal(got.cpu().numpy(), ref)
+    # two-stage linking: outliers of a tighter linking, grown with the relaxed criteria
+    ell = rng.uniform(1.5, 4.0, n).astype(np.float32)
+    prm = np.array([250.0 ** 2, 60.0 ** 2, 0, 0, 0])
+    hs2 = np.zeros((1, 12))
+    hs2[0, :3] = [0, n, 1]
+    hs2[0, 9:11] = prm[:2]
+    args = dict(v_ratio=3.0, theta_op=1.2)
+    P = Params.default(nsearch_min=20, nmin=4, **args)
+    l6 = ctx.fof6d(_dev(pos), _dev(vel), _dev(ell), _dev(lab), _dev(hs2), P)
+    ctx.sync()
+    one = oracle.fof6d_halo(up, vel, m, (ell >= 2.5).astype(np.uint8), prm, nmin=4, **args)
+    assert np.array_equal(l6.cpu().numpy(), one)
+    ctx.grow_groups(_dev(pos), _dev(vel), _dev(ell), _dev(lab), _dev(hs2), l6, P, GrowParams.default())
+    ctx.sync()
+    two = oracle.grow_halo(up, vel, m, ell, one, prm, ell_th=2.5, **args)
+    assert np.array_equal(l6.cpu().numpy(), two)
