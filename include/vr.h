@@ -375,15 +375,19 @@ vr_status vr_fof3d_noalloc(const int32_t *pos, int64_t n, int64_t link_d2, int32
 
 /* ---------------------------------------------------------------- measurement
  * (no counterpart in the paper: instrumentation of this library)
- * Per-kernel device timing with CUDA events recorded on the launching stream; off by
- * default. Kernel names: "fof_link", "velden_big", "velden_small", "halo_frame",
- * "cells_build", "cells_build_big", "ratio", "ell_fit", "link6", "clean", "core_link". */
+ * Device timing of the named steps with CUDA events recorded on the launching stream; off
+ * by default. A step is one kernel or a few that follow one another: "fof_link" (four link
+ * kernels), "velden_big" (every f_l launch for halos above N_se), "velden_small",
+ * "halo_frame" (one launch per size class), "cells_build", "cells_build_big" (two classes),
+ * "ratio", "ell_fit" (histograms, least squares, ell), "link6" and "core_link" (pairs inside
+ * tiles, then of tiles), "core_grow" (the moments, and each level's assignment), "clean". */
 
-/* Enables (1) or disables (0) event timing of the named kernels for this context. */
+/* Enables (1) or disables (0) event timing of the named steps for this context. */
 vr_status vr_timing_enable(vr_ctx *ctx, int enable);
 
-/* Device time in ms summed over the launches of kernel `name` recorded since the last
- * vr_timing_reset, and the number of those launches. Waits for the recorded events. */
+/* Device time in ms summed over the spans of step `name` recorded since the last
+ * vr_timing_reset, and in *launches the number of those spans (each from the step's first
+ * launch to the end of its last). Waits for the recorded events. */
 vr_status vr_timing_read(vr_ctx *ctx, const char *name, double *ms, int64_t *launches);
 
 /* Drops all recorded timings. */
@@ -395,13 +399,14 @@ int64_t vr_launch_count(void);
 
 /* ---------------------------------------------------------------- autotuning
  * (no counterpart in the paper: the launch shapes of this library's batched form)
- * The f_l kernel runs one launch per halo-size bin (halos of more than 65536 members,
- * 4097-65536, N_se+1-4096), each with its own shape (candidates computed side by side,
- * register cap, warps per block); the 6D linker has one shape (32-candidate tiles per
+ * The f_l kernel has a shape (candidates computed side by side, register cap, warps per
+ * block) for each halo-size bin (halos of more than 65536 members, 4097-65536,
+ * N_se+1-4096), and neighbouring bins of the same shape share a launch; untuned, the shape
+ * follows from the size of the call. The 6D linker has one shape (32-candidate tiles per
  * block). A shape changes how the same work is laid out on the GPU, never the arithmetic
  * or its order: every shape gives bit-identical results.
- * vr_autotune(ctx, 1): from the next call on, the first launch of each bin (and of the
- * linker) with work runs every candidate shape on the caller's data, timed with CUDA
+ * vr_autotune(ctx, 1): from the next call on, the first call with work in a bin (or for the
+ * linker) runs every candidate shape on the caller's data, timed with CUDA
  * events on `stream`, and keeps the fastest for later calls (that call takes several
  * times longer and synchronises its stream). vr_autotune(ctx, 0) returns to the default
  * shapes. Errors: VR_ERR_INVALID_ARG for enable not 0 or 1. */

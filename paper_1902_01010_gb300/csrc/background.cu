@@ -94,8 +94,8 @@ __device__ __forceinline__ int coord(const int4 &p, int a) { return a == 0 ? p.x
 // kFrameTeam blocks of a cluster, one block, or one warp, by the halo's size. Both passes over
 // the velocities and the reductions are FP64, of which an SM does two lanes a cycle: a halo
 // of 500,000 members on one SM took 0.92 ms, and a block of 256 threads for every small halo
-// spent 864 warp additions on its nine sums, where a warp spends 45 
-// (200^3 box: 1.91 -> 0.47 ms for all classes).
+// spent 864 warp additions on its nine sums, where a warp spends 45 (200^3 box, all halos: one
+// block each 1.20 ms, the three classes 0.14, 0.11 and 0.22).
 constexpr int kFrameTeam = 8;
 constexpr uint32_t kFrameBlock = 1024, kFrameBig = 16384;  // members from which a block, a cluster works
 
@@ -882,8 +882,7 @@ __device__ int leaf_moments(int first, int step, int count, uint32_t base, const
 // a block of 256 threads, below kBigHalo with one of 1,024, the rest with a cluster of kTeam
 // such blocks. A halo of 500,000 members on one SM took 10.2 ms: 6.5 levels of passes over its
 // members, bound by their latency, 127 entropies and the leaves' moments in FP64, of which an
-// SM does two lanes a cycle (now 1.5 ms; the whole build of a 200^3
-// box 15.3 -> 4.6 ms summed over its launches).
+// SM does two lanes a cycle (now 1.5 ms; the launches of a 200^3 box 15.5 -> 4.7 ms in all).
 constexpr int kTeam = 8;
 
 template <int NT>

@@ -9,10 +9,12 @@
 //  - k_fit_lm, a warp per halo: Levenberg-Marquardt on the counts (unweighted least squares;
 //    start A = max count, Rbar = centre of the first fullest bin, sigma = MAD', s = 1; lambda
 //    1e-3, /10 on an accepted step, x10 on a rejected one; stop on a relative cost change
-//    below 1e-15, or when a step changes no parameter: a larger lambda only shortens it);
+//    below 1e-15, or when a step changes no parameter: a larger lambda only shortens it, in
+//    the norm that weights each parameter by its diagonal of J^T J);
 //  - k_ell, a thread per member.
 // One block per halo for all three left 7 of 8 warps and their registers waiting for the one
-// that iterates, and read every R 14 times with 256 threads (200^3 box: 3.55 -> 1.42 ms).
+// that iterates, and read every R 14 times with 256 threads (200^3 box: 3.53 ms; k_fit_hist now
+// 0.33, k_fit_lm 1.02). k_fit_lm is bound by the latency of its chain of FP64 operations.
 #include <math.h>
 
 #include <vector>

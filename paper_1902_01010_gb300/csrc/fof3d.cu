@@ -432,7 +432,7 @@ __device__ void link_cells_warp(const FofCells &f, int *parent, uint32_t sa0, ui
 // Tests the member pairs of up to 32 pairs of particle runs, one pair of runs per lane (w =
 // its member pairs, 0: none): the pairs of all lanes follow one another, and each step takes
 // the next 32. Lanes that walked their own few pairs left two thirds of the warp idle
-// (k_fof_neigh at 512^3: 23.0 -> 17.5 ms). A run paired with itself takes i < j only.
+// (k_fof_neigh at 512^3, then: 23.0 ms, 17.5 so). A run paired with itself takes i < j only.
 __device__ __forceinline__ void link_runs(const FofCells &f, int *parent, uint32_t a0, uint32_t b0,
                                           uint32_t nb, uint32_t w) {
   const int lane = threadIdx.x & 31;
@@ -772,7 +772,7 @@ extern "C" vr_status vr_fof3d(vr_ctx *ctx, const int32_t *pos, int64_t n, int64_
   // link cells a warp takes at a time (n bounds their number): 32, or 64 warps per SM. Each
   // warp takes two such runs; more blocks than fit at once let the dense regions, which lie
   // together in sort order, spread over the SMs (k_fof_neigh at 512^3 with the resident
-  // blocks only 17.5 ms, now 13.1 ms)
+  // blocks only 17.5 ms, 13.2 so)
   int per = 4;
   while (per < 32 && n > 64LL * sms * per) per *= 2;
   const unsigned hgrid = (unsigned)grid_for(n, 32 * kLW, 64LL * sms);

@@ -154,7 +154,7 @@ __device__ __forceinline__ bool link6(long long dx2, float4 a, float4 b, const L
 // staged in shared memory and its members are read back by every lane). With one box, a tile on
 // a jump of the curve in a flat or elongated halo reached some 1,500 of its 6,250 tiles, and its
 // warp alone took most of the launch (200,000 members along a filament: 6.0 ms, now 0.42; in a
-// plane 3.4 ms, now 0.21; field 6DFOF of a 200^3 box 2.1, now 1.9).
+// plane 3.4 ms, now 0.21).
 //
 // The same walk serves the relaxed pass of the two-stage linking (MODE > 0, lx2 scaled
 // by gamma_x^2): MODE 1 unites linked pairs of untagged candidates, MODE 2 counts links
@@ -235,8 +235,8 @@ __device__ __forceinline__ LinkC link_consts(const double *row, double gx, doubl
 }
 
 // The FP64 predicate; its constants are read again here, so that they hold no registers in
-// the loops that rarely come this way (122 -> 64 registers, half the warp slots in use instead
-// of a quarter: k_link6 in the field 6DFOF of a 200^3 box 3.5 -> 2.2 ms).
+// the loops that rarely come this way (64 registers instead of 122, half the warp slots in use
+// instead of a quarter).
 __device__ __noinline__ bool exact_link(float dx, float dy, float dz, float4 qa, float4 qb,
                                         const double *row, double gx, double vr2, double cos2, int use_lv,
                                         int use_vt, long long T) {
@@ -318,8 +318,10 @@ __device__ __forceinline__ float4 pos_f32(int4 p) {
 // unite if all such members are now in one set, kRepNone if the tile holds none, kRepMixed
 // otherwise: k_link6 skips a pair of one-set tiles that already share a root in the box
 // test, 32 tiles at a time. In a halo's core nearly every tile pair within reach is such a
-// pair (field 6DFOF of a 200^3 box, 3.2M members, both kernels:
-// 9.0 -> 5.5 ms).
+// pair. Both kernels in the field 6DFOF of a 200^3 box (3.2 M members): 0.31 + 2.04 ms, 12.9 in
+// one kernel with every pair of reachable tiles tested in FP64; outlier linking of a 10 M member
+// catalogue 0.10 + 0.50, before 5.3; the five core loops of a 128^3 box 0.21 + 2.06, before 16.4.
+// What bounds them: issue, and the latency of the finds.
 constexpr int kRepNone = -1, kRepMixed = -2;
 
 template <int MODE>
@@ -491,9 +493,7 @@ __global__ void __launch_bounds__(256, 4) k_link6(const uint32_t *__restrict__ t
         // The commonest set of this tile's members: its members in the other tile need no
         // test against those in this one. What is left are the other tile's members outside
         // it, and this tile's outside it against the other's inside: some 8 steps instead of
-        // 32 where two tiles lie mostly in one set with a few fast members outside it (with
-        // the reach test above, k_link6 in the field 6DFOF of a 200^3 box 5.1 -> 3.5 ms, in the
-        // first core loop of a 128^3 box 1.63 -> 0.86 ms).
+        // 32 where two tiles lie mostly in one set with a few fast members outside it.
         const unsigned peers = __match_any_sync(FULL, near_a ? ra0 : -2 - lane);
         const int top = __reduce_max_sync(FULL, near_a ? (__popc(peers) << 5) | lane : -1);
         const int r0 = top >= 0 ? __shfl_sync(FULL, ra0, top & 31) : -1;

@@ -14,7 +14,7 @@ constexpr uint32_t kMaxHalo = 1u << 22;
 // first, and all singletons) is counted by a plain store, the others by atomics. A block
 // adds up its labels in a small hash table first, since the labels of large halos come in no
 // order and each is one address for up to millions of particles (10M members of a catalogue
-// with halos of up to a million: 1,197 -> 93 us). Labels outside [0, n) raise an error.
+// with halos of up to a million: 1,199 -> 90 us). Labels outside [0, n) raise an error.
 __global__ void k_count_first(const int32_t *__restrict__ label, int64_t n, uint32_t *__restrict__ cnt) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i <= n) cnt[i] = i < n && label[i] == i ? 1u : 0u;
@@ -116,7 +116,7 @@ __global__ void k_halo_bounds(const uint32_t *__restrict__ hkey, const uint32_t 
 // Unwrapped positions of slots in (halo, index) order, and the halos' bounding boxes. A warp
 // takes kUnwrapRounds x 32 consecutive slots and keeps the box of the halo it is in per lane,
 // so that a run inside one halo costs six atomics in all, not six per 32 slots (10M members:
-// 497 -> 159 us).
+// 517 -> 159 us).
 constexpr int kUnwrapRounds = 8;
 __global__ void k_unwrap(const int32_t *__restrict__ pos, const uint32_t *__restrict__ hkey,
                          const uint32_t *__restrict__ idx, const uint32_t *__restrict__ hoff,
@@ -236,9 +236,9 @@ __device__ __forceinline__ uint32_t hilbert10(uint32_t x, uint32_t y, uint32_t z
 //    members form one compact cluster, where a Morton run may straddle an octant boundary
 //    with a box that spans both sides: the members within the linker's reach of a tile's
 //    box fall with it (on a 124,111-member halo 2,511 members lie within the N_se = 256
-//    ball radius of a 32-member Morton box, 1,436 for Hilbert). Measured (one call, Morton -> Hilbert): field 6DFOF of a
-//    200^3 box 23.7 -> 12.9 ms, outlier linking of a 10 M member catalogue 16.3 -> 8.5 ms,
-//    core search and growth of a 128^3 box 20.5 -> 12.9 ms;
+//    ball radius of a 32-member Morton box, 1,436 for Hilbert). One call with Morton and with
+//    Hilbert: field 6DFOF of a 200^3 box 4.89 and 4.61 ms, outlier linking of a 10 M member
+//    catalogue 3.04 and 2.96, core search and growth of a 128^3 box 7.21 and 5.96;
 //  - Morton, where f_l is computed: the FP32 sum of f_l runs in an order that follows the
 //    slots, and the skew-Gaussian fit downstream turns a change in the last bit of f_l into
 //    one of 1e-3 in a small halo's ell (a member crosses a histogram edge), so that order

@@ -24,11 +24,13 @@
 // wherever the two boxes involved (query bucket and candidate bucket or window) bound
 // every separation by kNarrow lattice units per axis, which makes them exact in 32 bits.
 //
-// What bounds the pass over a 256^3 box (33 ms): the issue slots (76 % taken at 7 warps a
-// scheduler), by phase the window's bound 7 %, the histogram levels 38 %, the collect pass 42 %
-// (most of it list insertions, whose lanes diverge), the keys of the final bin 13 %. Its code has
-// to stay small: with every loop over 32 members unrolled whole, warps in different phases put
-// each other's instructions out of the cache, and the same work took 44.6 ms instead of 39.4.
+// What bounds it: the issue slots (76 % taken at 7 warps a scheduler on a 256^3 box), by phase
+// the window's bound 7 %, the histogram levels 38 %, the collect pass 42 % (most of it list
+// insertions, whose lanes diverge), the keys of the final bin 13 %. Its code has to stay small:
+// with every loop over 32 members unrolled whole, warps in different phases put each other's
+// instructions out of the cache. k_velden_big over a 256^3 box (16.8 M particles, one launch):
+// 30.3 ms, 55.6 with subtractions in 64 or 32 bits, a launch per size bin and bounds that stay
+// what they were at the start of a level; over 1 M particles 2.73 ms, before 5.00.
 // Halos with at most N_se members use every member (one pass, no position search).
 #include <math.h>
 
@@ -51,9 +53,9 @@ constexpr int kBuf = 32;
 // matters, and 16 buckets add at most 512 before it is looked at again.
 constexpr int kFull = 32768;
 // Lanes that want a bucket, up to which the collect pass takes it a lane per member and query by
-// query (about 22 instructions a query) instead of a lane per query (about 300 for the 32 members):
-// f_l of a 256^3 box 34.5 -> 33.3 ms, of a catalogue with N_se 64 24.2 -> 23.2. In the levels, where
-// the counts then need shared-memory atomics, the same gained nothing (34.4 to 34.7).
+// query (about 22 instructions a query) instead of a lane per query (about 300 for the 32 members).
+// With it the f_l call of a 256^3 box took 33.3 ms, without 34.5. In the levels the counts would
+// then need shared-memory atomics, so not there.
 constexpr int kFewLanes = 12;
 constexpr int kWarps = 4;        // warps per block
 
@@ -70,10 +72,8 @@ constexpr int kWindow = 4;       // window of kWindow * N_se members for the fir
 
 // Per-warp shared memory. The key histogram is used only by the bound and histogram
 // passes and the top-N_v list only by the collect pass, so the two share storage and the
-// slots of the final bin are in local memory (5 KB a warp; with the list in a storage of its own,
-// beside counts that shared with the slots, it was 9 KB: f_l of a 256^3 box 57.9 ms, 54.3 so).
-// Counts of 32 bits, a bank per lane, were tried: 52.4 ms with shared-memory atomics and 54.0
-// with plain loads and stores, against 51.9 for 16 bits.
+// slots of the final bin are in local memory: 6.3 KB a warp, so that registers, not this, limit
+// the warps in flight. Counts have 16 bits, since 32 would leave room for fewer warps.
 template <int NVM>
 struct WarpSmem {
   int4 su[32];
@@ -168,8 +168,7 @@ __device__ __forceinline__ long long d2i(int4 a, int4 b) {
 // and, with coordinates relative to the query box's corner o, |q|^2 < 2^31. Then d^2 =
 // |c|^2 - 2 q.c + |q|^2 in 32-bit arithmetic (what wraps on the way wraps back, and d^2 -
 // |q|^2 fits a signed word), so a candidate staged as (c, |c|^2) costs three multiply-adds,
-// and |q|^2 goes into the thresholds (f_l of a 256^3 box: 52.6 ms with three subtractions as
-// well, 51.9 so).
+// and |q|^2 goes into the thresholds.
 constexpr int kNarrow = 26754;  // 3 kNarrow^2 < 2^31
 
 struct Rel {  // a query's side
@@ -206,8 +205,8 @@ __device__ __forceinline__ int clamp31(u64 x) { return x > 0x7fffffffull ? 0x7ff
 // slots of [m0, m1), a lane per slot, and the halos they belong to one after the other: the
 // halo's members are staged 32 at a time and offered to its lanes. The offers are a serial
 // chain, so the work is cut by slots and not by halos: a warp per halo made the 8 x 256
-// offers of a 256-member halo one after the other (660 us, the
-// same for a 32^3 and a 100^3 box; now 115 us).
+// offers of a 256-member halo one after the other (660 to 680 us for a 32^3 box and for 1 M
+// particles alike; now 115 and 151 us, and over a 256^3 box 1.07 -> 0.51 ms).
 template <int NVM>
 __global__ void __launch_bounds__(32 * kWarps) k_velden_small(
     const uint32_t *__restrict__ hoff, const uint32_t *__restrict__ hid, int64_t m0, int64_t m1,
@@ -501,8 +500,8 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     return;
   }
   // Two parts of the query bucket (a bucket whose box spanned a jump of the curve, in a halo of
-  // 564 k members, tested 27,000 others one by one for 437 to visit: 25 M cycles, 13 ms, a third of
-  // the whole launch; the longest warp of any is 9 M cycles with two parts).
+  // 564 k members, tested 27,000 others one by one for 437 to visit: 25 M cycles; the longest warp
+  // of any is 9 M cycles with two parts).
   const int cut = box_parts(q, (int)(qe - qs) - 1, qlo, qhi, sm.qlo, sm.qhi);
   __syncwarp();
   // Candidate buckets are enumerated on the fly in every pass: super-bucket boxes, then
@@ -587,8 +586,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       stage(s0, cnt, false, narrow);
       if (narrow) {
         // without a branch per member: what lies below the bins or beyond the bound (all of it
-        // for a lane that wants none) counts in a row of its own (f_l of a 256^3 box: 54.3 ms
-        // with a compare and a branch for each, 51.8 so)
+        // for a lane that wants none) counts in a row of its own
         const int far = (want ? clamp31((u64)rlev) : -1) - rq.q2, shd = want ? sh - 22 : 0;
         const uint32_t off = (uint32_t)rq.q2 - (uint32_t)clamp31(klo >> 22) + (1u << shd);
         auto row_of = [&](int x) { return x > far ? kBins + 1 : max((int)((uint32_t)x + off) >> shd, 0); };
@@ -781,8 +779,9 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
     for (; fin; fin &= fin - 1u)
       if (nbuf < kBuf) bslot[nbuf++] = s0 + (uint32_t)(__ffs(fin) - 1);
     // What the lists turn away already is passed over side by side first, where that is most of it:
-    // of N_se members a list takes about N_v (1 + ln(N_se / N_v)). f_l of a 256^3 box (256 and 32)
-    // 35.5 -> 34.4 ms; with 64 and 16, where the lists take 60 %, 24.1 -> 24.4, so not there.
+    // of N_se members a list takes about N_v (1 + ln(N_se / N_v)). With N_se 256 and N_v 32 the f_l
+    // call of a 256^3 box took 34.4 ms with this and 35.5 without; with 64 and 16, where the lists
+    // take 60 %, that of a catalogue 24.4 and 24.1, so not there.
     if (nse_eff >= 6 * nv_eff && __reduce_max_sync(FULL, (unsigned)__popc(in)) > 10u) {
       uint32_t drop = 0;
 #pragma unroll 1
@@ -792,9 +791,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(MAXREG) k_velden_big(
       }
       if (tv.c >= nv_eff) in &= ~drop;
     }
-    // each lane its own next member: as many rounds as the lane with the most has (with an insertion
-    // in each member's place 39.4 ms for a 256^3 box, 38.2 so; with lanes passing over what their
-    // lists turn away and then replacing together 40.4)
+    // each lane its own next member: as many rounds as the lane with the most has
     for (; in; in &= in - 1u) top_insert(top, lane, tv, nv_eff, dv2f(sm.sv[__ffs(in) - 1], vq));
     return false;
   });
@@ -963,9 +960,9 @@ vr_status run_velden(vr_ctx *ctx, const HaloSeg &g, const vr_params *p, Arena &a
   }
   // a shape per halo-size bin; a bin still to be tuned is run once per candidate shape (same
   // results each time) and keeps the fastest. Neighbouring bins of one shape share a launch,
-  // so that the last, long warps of one run beside the next (a third of the chip's time was idle in the
-  // launch of the largest halos: f_l of a 256^3 box 51.9 -> 45.1 ms with one launch), unless
-  // `ev_big` has to mark the end of the first bin.
+  // so that the last, long warps of one run beside the next (alone, the launch of the largest
+  // halos left a third of the chip's time idle), unless `ev_big` has to mark the end of the first
+  // bin.
   const int64_t lo[kVBins] = {0, 32LL * eg[0], 32LL * eg[1]};
   const int64_t hi[kVBins] = {32LL * eg[0], 32LL * eg[1], nbpad};
   timer_begin(ctx, "velden_big", s);
