@@ -162,12 +162,12 @@ def measured_peaks():
 # Epanechnikov sum over N_v (3 ops): 256*8 + 256*8 + 256 + 256 + 32*3 = 4,704 ALU ops.
 VELDEN_OPS_PER_QUERY = 256 * 8 + 256 * 8 + 256 + 256 + 32 * 3
 # DRAM bytes per query particle of k_velden_big from one ncu capture (dram__bytes_read.sum
-# + dram__bytes_write.sum of one launch over its query particles); the kernel's traffic
-# grows with its queries, so a full launch is this times its queries. None whenever the
-# kernel has changed since the capture.
-VELDEN_DRAM_BYTES_PER_QUERY = 12800662784 / 39635926
-VELDEN_DRAM_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the two "
-                      "k_velden_big launches of one 512^3 step (12.80 GB over 39,635,926 query "
+# + dram__bytes_write.sum of one launch over its query particles) on a 200^3 box; the kernel's
+# traffic grows with its queries, so a full launch is estimated as this times its queries. None
+# whenever the kernel has changed since the capture.
+VELDEN_DRAM_BYTES_PER_QUERY = 586492928 / 2256982
+VELDEN_DRAM_SOURCE = ("estimate: ncu dram__bytes_read.sum + dram__bytes_write.sum of one "
+                      "k_velden_big launch on a 200^3 box (586 MB over 2,256,982 query "
                       "particles), times this step's query particles")
 LANES_PER_SM = 128  # FP32/INT32 lanes per SM (4 partitions x 32)
 
@@ -504,7 +504,7 @@ def run_ours(args):
                                f"{sm_mhz:.0f} MHz (sm_max_mhz of {how} peaks): one 32-bit "
                                f"operation per lane per clock",
                 "algorithmic": f"{VELDEN_OPS_PER_QUERY} ops x {int(nq_big)} query particles",
-                "launch_ms": per_launch_ms,
+                "launch_ms": per_launch_ms,  # all of the step's k_velden_big launches
                 "hbm_achieved_gbs": kern_b["velden_big"] / (per_launch_ms / 1e3) / 1e9,
                 "hbm_frac": kern_b["velden_big"] / (per_launch_ms / 1e3) / 1e9 / hbm}
     elif dom == "fof_link" and kern[dom][1] > 0:
